@@ -703,8 +703,9 @@ static cudaError_t enqueue_sum(cs_ctx* ctx, const LikPlan& L, const float* img,
     cudaError_t e;
     {
         StageTimer tm(ctx, CS_STAGE_GATHER, st);
+        // (the smooth texture has representatives of its own)
         e = launch_gather(img, L.H, L.W, bitmask, L.k, L.n_labels, L.d_off, sample_pix, L.S,
-                          !L.persample, L.t, st);
+                          prm->mode == CS_MODE_FACTORISED, L.t, st);
         if (e == cudaSuccess && L.tc_form) e = launch_sum_tc_prepare(T, sorted, st);
     }
     if (e == cudaSuccess && dist_ready) e = cudaStreamWaitEvent(st, dist_ready, 0);
