@@ -295,8 +295,10 @@ cs_status cs_kmedians(cs_ctx* ctx, const float* V, int N, int k, int n_classes,
     if (!s) s = unsup_init(ctx, fn, init, n_classes, N, &in);
     if (s) return s;
     DeviceGuard g(ctx->device);
-    if (!assign && (s = cs_ensure_scratch(ctx, sizeof(int32_t) * (size_t)N))) return s;
-    int32_t* work = assign ? assign : reinterpret_cast<int32_t*>(ctx->scratch);
+    // the rounds' assignments, one byte each: the result's memory holds them
+    // until the last assignment overwrites it
+    if (!assign && (s = cs_ensure_scratch(ctx, (size_t)N))) return s;
+    uint8_t* work = reinterpret_cast<uint8_t*>(assign ? (void*)assign : (void*)ctx->scratch);
     KmediansArgs a{V, N, k, n_classes, in, iterations, centres, assign, work, ctx->n_sm};
     cudaError_t e = launch_kmedians(a, (cudaStream_t)stream);
     if (e != cudaSuccess) return cs_set_error(ctx, CS_ERR_CUDA, "%s: %s", fn, cudaGetErrorString(e));
@@ -343,32 +345,41 @@ cs_status cs_unsup_data_term(cs_ctx* ctx, const float* img, int H, int W, const 
                             up->n_colour, up->n_texture, CS_MAX_LABELS);
     DeviceGuard g(ctx->device);
     const int nc = up->n_colour, nt = up->n_texture;
-    auto carve = [&](Carve& c, float** iota, float** cc, float** tc, void** km, int32_t** work) {
+    auto carve = [&](Carve& c, float** iota, float** cc, float** tc, void** km, uint8_t** work) {
         *iota = c.take<float>((size_t)k * P);
         *cc = colour_centres ? colour_centres : c.take<float>(3 * (size_t)nc);
         *tc = texture_centres ? texture_centres : c.take<float>((size_t)nt * k);
         *km = c.take<char>(kmeans_scratch_bytes(nc));
-        *work = texture_assign ? texture_assign : c.take<int32_t>(P);
+        uint8_t* own = c.take<uint8_t>(texture_assign ? 0 : P);
+        *work = texture_assign ? reinterpret_cast<uint8_t*>(texture_assign) : own;
     };
     float *iota, *cc, *tc;
     void* km;
-    int32_t* work;
+    uint8_t* work;
     Carve m(nullptr);
     carve(m, &iota, &cc, &tc, &km, &work);
     if ((s = cs_ensure_scratch(ctx, m.off))) return s;
     Carve c(ctx->scratch);
     carve(c, &iota, &cc, &tc, &km, &work);
     cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e = launch_iota_pixels(img, H, W, omega, k, prm->p, mask, (float)prm->iota_sigma,
-                                       iota, st);
+    // the colour clustering needs only the image: it runs on the context's side
+    // stream under the texture clustering (joined also after an error)
+    cudaError_t e = cudaEventRecord(ctx->ev_fork, st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
     if (e == cudaSuccess) {
         KmeansArgs a{img, (int)P, nc, ci, up->kmeans_iterations, cc, nullptr, km, ctx->n_sm};
-        e = launch_kmeans(a, st);
-    }
-    if (e == cudaSuccess) {
-        KmediansArgs a{iota, (int)P, k, nt, ti, up->kmedians_iterations, tc, nullptr, work,
-                       ctx->n_sm};
-        e = launch_kmedians(a, st);
+        e = launch_kmeans(a, ctx->side);
+        cudaError_t e2 = launch_iota_pixels(img, H, W, omega, k, prm->p, mask,
+                                            (float)prm->iota_sigma, iota, st);
+        if (e == cudaSuccess) e = e2;
+        if (e == cudaSuccess) {
+            KmediansArgs b{iota, (int)P, k, nt, ti, up->kmedians_iterations, tc, nullptr, work,
+                           ctx->n_sm};
+            e = launch_kmedians(b, st);
+        }
+        e2 = cudaEventRecord(ctx->ev_join, ctx->side);
+        if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(st, ctx->ev_join, 0);
+        if (e == cudaSuccess) e = e2;
     }
     if (e == cudaSuccess) {
         UnsupFinalArgs a{img, (int)P, iota, k, cc, nc, tc, nt, (float)(0.5 / prm->sigma_c2),

@@ -204,7 +204,6 @@ struct SegArgs {
 size_t seg_scratch_bytes(long long P, int n, int nblk);
 int seg_blocks(long long P, int n_labels, int n_sm);  // 0 if the kernel cannot be resident
 cudaError_t launch_segment(const SegArgs& a, cudaStream_t st);
-size_t smooth_smem_bytes(int p, int k, int n_labels);
 
 // Unsupervised mode (Sec. 3.2): iota of every pixel, clusterings, data term.
 cudaError_t launch_iota_pixels(const float* img, int H, int W, const float* omega, int k, int p,
@@ -230,7 +229,7 @@ struct KmediansArgs {
     int iterations;
     float* C;              // out: n x k
     int32_t* assign;       // out (optional): N
-    int32_t* work_assign;  // N (may equal assign)
+    uint8_t* work_assign;  // N bytes (may share assign's memory)
     int n_sm;
 };
 struct UnsupFinalArgs {
