@@ -161,7 +161,8 @@ cs_status cs_sync_status(cs_ctx* ctx, void* stream);
  *             CS_STALL_NONE     none (disarms a pending stall)
  *             CS_STALL_SEGMENT  cs_segment: the last block of the cooperative
  *                               launch skips its arrival at the first grid
- *                               barrier of the iterations (needs iterations > 0)
+ *                               barrier (or its first exchange) of the
+ *                               iterations (needs iterations > 0)
  *             CS_STALL_SUM      the tensor-core sum (cs_likelihood or
  *                               cs_data_term with CS_BF16 / CS_FP8): the
  *                               MMA-issuing thread of the last CTA waits,
@@ -327,9 +328,12 @@ cs_status cs_refined_count(cs_ctx* ctx, int32_t* count, void* stream);
  *              label on ties
  *   n_labels   1..64;  H W < 2^31
  * Defaults (cs_seg_params_default): lambda 1, nu 0, gamma 5, 300 iterations.
- * Uses the context's scratch (4 n P + P floats). Asynchronous on `stream`:
- * one cooperative launch runs every iteration, with grid barriers between
- * the dual and primal steps. Errors: CS_ERR_INVALID_ARG for null or
+ * Uses the context's scratch (at most 4 n P + P floats). Asynchronous on
+ * `stream`: one cooperative launch runs every iteration. Up to 16 labels, images
+ * whose state fits the chip (about 150,000 pixels at 16 labels, 380,000 at 5)
+ * are split into one tile per SM that exchange their borders; larger ones keep
+ * the state in global memory, with grid barriers between the dual and primal
+ * steps. The two forms agree to rounding. Errors: CS_ERR_INVALID_ARG for null or
  * out-of-range arguments; CS_ERR_CUDA when the launch fails; a grid barrier
  * that waits longer than 1 s ends the launch and is reported as
  * CS_ERR_TIMEOUT by the next cs_sync_status.

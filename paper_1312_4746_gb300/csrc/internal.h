@@ -197,11 +197,12 @@ struct SegArgs {
     float* scratch;    // seg_scratch_bytes()
     int nblk;          // blocks of the cooperative launch (seg_blocks)
     int* d_err;        // device error word (timeout of a grid barrier)
+    int n_sm;
     unsigned long long wait_ns = 0;  // limit of each grid-barrier wait (0: 1 s)
     bool stall = false;  // timeout-path test: the last block skips its first arrival of
                          // the iterations
 };
-size_t seg_scratch_bytes(long long P, int n, int nblk);
+size_t seg_scratch_bytes(int H, int W, int n, int nblk, int n_sm, bool sums);
 int seg_blocks(long long P, int n_labels, int n_sm);  // 0 if the kernel cannot be resident
 cudaError_t launch_segment(const SegArgs& a, cudaStream_t st);
 
