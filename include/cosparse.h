@@ -56,7 +56,8 @@ typedef int cs_status;
                                 -||c_i - iota(O s_x)||_1 / beta_i(x); cs_data_term only */
 
 /* Arithmetic forms. */
-#define CS_FP32 0 /* CUDA-core FP32 with exact integer distances and popc TSM */
+#define CS_FP32 0 /* CUDA-core FP32 with exact integer distances; the TSM, an exact integer, from
+                     the tensor cores */
 #define CS_BF16 1 /* tensor-core (tcgen05) TSM, colour and location dot products, FP32 accumulation */
 #define CS_FP8 2  /* as CS_BF16 with FP8 operands where they are exact */
 

@@ -568,11 +568,13 @@ void cs_lik_plan(LikPlan& L, int H, int W, int k, int n_labels,
     L.offs.v[n_labels + 1] = 0;
     for (int i = 0; i < n_labels; ++i)
         L.offs.v[n_labels + 2 + i] =
-            L.offs.v[n_labels + 1 + i] + tc_tiles_per_label(label_off[i + 1] - label_off[i]);
+            L.offs.v[n_labels + 1 + i] + (L.tc_form ? tc_tiles_per_label(label_off[i + 1] - label_off[i])
+                                                    : plain_tiles_per_label(label_off[i + 1] - label_off[i]));
     L.total_tiles = L.offs.v[2 * n_labels + 1];
     L.n_chunks = 0;
     for (int i = 0; i < n_labels; ++i) L.n_chunks += (label_off[i + 1] - label_off[i] + 4095) / 4096;
-    L.stage_bytes = tc_copy_bytes(k, L.tex8, L.persample);
+    L.stage_bytes = L.tc_form ? tc_copy_bytes(k, L.tex8, L.persample)
+                              : plain_tile_bytes(k, L.persample);
 }
 
 void cs_lik_carve(Carve& c, LikPlan& L, int32_t* dist2) {
@@ -594,7 +596,7 @@ void cs_lik_carve(Carve& c, LikPlan& L, int32_t* dist2) {
     L.t.sbits = c.take<uint32_t>((size_t)Wk * S);
     L.t.spop = c.take<int32_t>(S);
     L.t.rep = c.take<uint32_t>((size_t)n * Wk);
-    L.t.blob = c.take<uint8_t>(L.tc_form ? (size_t)L.total_tiles * L.stage_bytes : 0, 1024);
+    L.t.blob = c.take<uint8_t>((size_t)L.total_tiles * L.stage_bytes, 1024);
     L.t.tile_xy = c.take<uint32_t>(L.tc_form ? (size_t)L.total_tiles * tc_tile_samples() : 0);
     L.t.perm = c.take<int32_t>(L.tc_form ? (size_t)S : 0);
     L.desc = c.take<TcImage>(L.tc_form ? 1 : 0);
@@ -624,7 +626,7 @@ static cudaError_t enqueue_distances(cs_ctx* ctx, const LikPlan& L, const int32_
     return launch_edt(ea, st);
 }
 
-SumArgs cs_sum_args(const LikPlan& L, const float* img, const uint32_t* bitmask,
+SumArgs cs_sum_args(cs_ctx* ctx, const LikPlan& L, const float* img, const uint32_t* bitmask,
                     const cs_params* prm, float* neglog, float* post) {
     SumArgs a{};
     a.img = img;
@@ -646,6 +648,7 @@ SumArgs cs_sum_args(const LikPlan& L, const float* img, const uint32_t* bitmask,
     a.rho_var = prm->rho_variance != 0;
     a.neglog = neglog;
     a.post = post;
+    a.d_err = ctx->d_err;
     return a;
 }
 
@@ -718,12 +721,15 @@ static cudaError_t enqueue_sum(cs_ctx* ctx, const LikPlan& L, const float* img,
         // (the smooth texture has representatives of its own)
         e = launch_gather(img, L.H, L.W, bitmask, L.k, L.n_labels, L.d_off, sample_pix, L.S,
                           prm->mode == CS_MODE_FACTORISED, L.t, st);
-        if (e == cudaSuccess && L.tc_form) e = launch_sum_tc_prepare(T, sorted, st);
+        if (e == cudaSuccess)
+            e = L.tc_form ? launch_sum_tc_prepare(T, sorted, st)
+                          : launch_plain_tiles(L.d_off, L.n_labels, L.total_tiles, L.k, L.S,
+                                               L.persample, L.t, st);
     }
     if (e == cudaSuccess && dist_ready) e = cudaStreamWaitEvent(st, dist_ready, 0);
     if (e != cudaSuccess) return e;
     StageTimer tm(ctx, CS_STAGE_SUM, st);
-    if (!L.tc_form) return launch_sum_plain(cs_sum_args(L, img, bitmask, prm, neglog, post), st);
+    if (!L.tc_form) return launch_sum_plain(cs_sum_args(ctx, L, img, bitmask, prm, neglog, post), st);
     return launch_sum_tc_run(T, st);
 }
 
@@ -805,15 +811,17 @@ cs_status cs_plan_likelihood(cs_ctx* ctx, LikPlan& L, int H, int W, int k, int n
     return CS_OK;
 }
 
-// distances and sample tables
+// distances, sample tables and the plain form's sample tiles
 cudaError_t cs_enqueue_prepare(cs_ctx* ctx, const LikPlan& L, const float* img,
                                const uint32_t* bitmask, const int32_t* sample_pix,
                                const cs_params* prm, cudaStream_t st) {
     cudaError_t e = enqueue_distances(ctx, L, sample_pix, st);
     if (e != cudaSuccess) return e;
     StageTimer tm(ctx, CS_STAGE_GATHER, st);
-    return launch_gather(img, L.H, L.W, bitmask, L.k, L.n_labels, L.d_off, sample_pix, L.S,
-                         prm->mode == CS_MODE_FACTORISED, L.t, st);
+    e = launch_gather(img, L.H, L.W, bitmask, L.k, L.n_labels, L.d_off, sample_pix, L.S,
+                      prm->mode == CS_MODE_FACTORISED, L.t, st);
+    if (e != cudaSuccess || L.tc_form) return e;
+    return launch_plain_tiles(L.d_off, L.n_labels, L.total_tiles, L.k, L.S, L.persample, L.t, st);
 }
 
 // exact plain sum over a device pixel list (after cs_enqueue_prepare): with
@@ -823,7 +831,7 @@ cudaError_t cs_enqueue_exact_list_prepared(cs_ctx* ctx, const LikPlan& L, const 
                                            const int32_t* list, const int* count, int cap,
                                            float* T_out, float* neglog, float* post,
                                            cudaStream_t st) {
-    SumArgs a = cs_sum_args(L, img, bitmask, prm, neglog, post);
+    SumArgs a = cs_sum_args(ctx, L, img, bitmask, prm, neglog, post);
     a.pix_list = list;
     a.list_count = count;
     a.list_cap = cap;

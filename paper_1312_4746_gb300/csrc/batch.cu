@@ -172,8 +172,10 @@ static cudaError_t enqueue_run(cs_batch* b, cudaStream_t st) {
             T.first_ptile = b->first_ptile[s];
             e = launch_tc_prepare(T, ss);
         } else {
-            e = launch_sum_plain(cs_sum_args(L, m.d.img, m.codes.bitmask, &b->prm, m.d.neglog,
-                                             m.d.post), ss);
+            e = launch_plain_tiles(L.d_off, L.n_labels, L.total_tiles, L.k, L.S, L.persample, L.t, ss);
+            if (e == cudaSuccess)
+                e = launch_sum_plain(cs_sum_args(ctx, L, m.d.img, m.codes.bitmask, &b->prm,
+                                                 m.d.neglog, m.d.post), ss);
         }
     }
     for (int j = 0; j < S; ++j) {

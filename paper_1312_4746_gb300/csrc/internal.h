@@ -270,7 +270,7 @@ struct SampleTables {
     uint32_t* sbits;  // word-major: [Wk][S]
     int32_t* spop;    // popcount of each sample's bitmask
     uint32_t* rep;    // [n_labels][Wk]
-    uint8_t* blob;    // tensor-core sample tiles (ring-stage layout)
+    uint8_t* blob;    // sample tiles (tensor-core form: ring-stage layout)
     uint32_t* tile_xy;  // tensor-core tile slots: sample position x | y << 16
     int32_t* perm;    // tensor-core sample order (Morton order in chunks of 4096)
 };
@@ -301,8 +301,16 @@ struct SumArgs {
     const int* list_count = nullptr;
     int list_cap = 0;
     float* T_out = nullptr;
+    int* d_err = nullptr;  // device error word (a wait for the tensor cores that gave up)
 };
+// (over the sample tiles of launch_plain_tiles, whose offsets per label follow
+// the label offsets at d_label_off + n_labels + 1)
 cudaError_t launch_sum_plain(const SumArgs& a, cudaStream_t st);
+int plain_tiles_per_label(int m);
+size_t plain_tile_bytes(int k, bool persample);
+cudaError_t launch_plain_tiles(const int32_t* d_label_off, int n_labels, int total_tiles, int k,
+                               int n_samples, bool persample, const SampleTables& t,
+                               cudaStream_t st);
 
 struct TcImage;
 
@@ -474,7 +482,7 @@ cs_status cs_check_codes_form(cs_ctx* ctx, const char* fn, const cs_params* prm,
 void cs_lik_plan(LikPlan& L, int H, int W, int k, int n_labels, const int32_t* label_off,
                         const cs_params* prm);
 void cs_lik_carve(Carve& c, LikPlan& L, int32_t* dist2);
-SumArgs cs_sum_args(const LikPlan& L, const float* img, const uint32_t* bitmask,
+SumArgs cs_sum_args(cs_ctx* ctx, const LikPlan& L, const float* img, const uint32_t* bitmask,
                     const cs_params* prm, float* neglog, float* post);
 TcLaunch cs_tc_launch(cs_ctx* ctx, const LikPlan& L, const float* img, const uint32_t* bitmask,
                       const int32_t* sample_pix, const cs_params* prm, float* neglog,
