@@ -20,9 +20,7 @@ SO = os.path.join(OUT, "libcosparse.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ARCH + [
     "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2", "--expt-relaxed-constexpr",
-    # one thread per kernel of a file: the solver's and the sum's instantiations
-    # would otherwise compile one after another (60 s against 20 s)
-    "-Xptxas", "-warn-spills", "--split-compile=0",
+    "-Xptxas", "-warn-spills",
 ]
 
 

@@ -49,24 +49,33 @@ __device__ __forceinline__ void guard_push(int2* guard, int cap, int* count, int
     if (idx < cap) guard[idx] = make_int2(pix, j);
 }
 
-// Thresholds codes j0 .. j0 + 15 of one pixel (from a tensor-memory load):
-// entry j (< k) goes to the co-support word when |a_j| <= tau and it is not
-// within its error bound E_j = rn_j ebase + slack of tau; entries within
-// the bound are marked in gword for the exact recheck. No branch per entry;
-// rn is zero-padded beyond k.
-__device__ __forceinline__ void threshold16(const uint32_t (&v)[16], int j0, int k, const float* rn,
+// Thresholds 16 consecutive codes of one pixel (from a tensor-memory load),
+// bits `sh` .. of a 32-code word: entry e goes to the co-support word when |a_e|
+// <= tau and it is not within its error bound E_e = rn_e ebase + slack of tau (d
+// = |a| - tau below -E); entries within the bound are marked in gword for the
+// exact recheck. No branch per entry. Entries beyond k are masked by the caller.
+__device__ __forceinline__ void threshold16(const uint32_t (&v)[16], int sh, const float* rn,
                                             float ebase, float tau_f, float tau_slack,
                                             uint32_t& word, uint32_t& gword) {
+    uint32_t w = 0, g = 0;
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        const int j = j0 + e;
-        const float aa = fabsf(__uint_as_float(v[e]));
-        const float E = rn[j] * ebase + tau_slack;
-        const bool g = fabsf(aa - tau_f) <= E;
-        const uint32_t m = j < k ? 1u << (j & 31) : 0u;
-        word |= (!g && aa <= tau_f) ? m : 0u;
-        gword |= g ? m : 0u;
+    for (int q = 0; q < 4; ++q) {
+        const float4 r = reinterpret_cast<const float4*>(rn)[q];
+        const float re[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float d = fabsf(__uint_as_float(v[4 * q + e])) - tau_f;
+            const float E = re[e] * ebase + tau_slack;
+            if (d < -E) w |= 1u << (4 * q + e);
+            if (fabsf(d) <= E) g |= 1u << (4 * q + e);
+        }
     }
+    word |= w << sh;
+    gword |= g << sh;
+}
+// bits of word w that are codes below k
+__device__ __forceinline__ uint32_t word_mask(int w, int k) {
+    return k - 32 * w >= 32 ? 0xffffffffu : (1u << (k - 32 * w)) - 1u;
 }
 
 // the guard entries of one 32-code word
@@ -194,27 +203,36 @@ __global__ void __launch_bounds__(TILE* TILE)
         for (int j = k; j < 16; ++j) lead16[(size_t)pix * 16 + j] = 0.f;
 }
 
-// Canonical double-precision recomputation of guarded entries, one warp per
-// entry (entries spread round-robin over the blocks, so over the SMs): the
-// patch and code follow the exact operation order of the definition (gray,
-// mask product, index-order sums, division by the square root), with every
-// operation correctly rounded and no contraction, so the result is
-// bit-identical to a sequential evaluation. The element-wise steps (pixel
-// loads, products, quotients) run across the lanes; only the three
-// index-order sums run on lane 0. An entry (pixel, j) decides code j;
-// (pixel, -1) every code of a nearly flat patch (one lane per code). Guarded
-// bits were left clear by the codes kernel and are set here.
+// Canonical double-precision recomputation of guarded entries. An entry (pixel,
+// j) decides code j; (pixel, -1) every code of a nearly flat patch. Guarded bits
+// were left clear by the codes kernel and are set here.
 //
-// A code entry is first decided from the same element values with warp-tree
-// sums, when that value is clear of tau by a bound that covers both it and
-// the index-order evaluation: from the values v_t (identical in both), with
-// u = 2^-53, A = sum |v_t|, ss = sum c_t^2, every mean, centring, square,
-// root, quotient, product and N-term sum is within
+// codes_guard_canonical: the patch and code follow the exact operation order of
+// the definition (gray, mask product, index-order sums, division by the square
+// root), with every operation correctly rounded and no contraction, so the
+// result is bit-identical to a sequential evaluation. One warp: the element-wise
+// steps (pixel loads, products, quotients) run across the lanes; only the three
+// index-order sums run on lane 0 (a flat patch: one lane per code).
+//
+// codes_guard_kernel first tries to decide an entry from the same element
+// values v_t with sums in another order: from these (identical in both), with u
+// = 2^-53, A = sum |v_t|, ss = sum c_t^2, every mean, centring, square, root,
+// quotient, product and N-term sum is within
 //   |a - a_exact| <= |O_j| (e_s + N u (1 + e_s)),
 //   e_s = 2 u sqrt(N) A / sqrt(ss) + (N / 2 + 5) u   (bound on |s - s_exact|)
-// of the exact value in either summation order, so the two differ by at most
-// twice that; the filter asks for four times (an entry closer to tau, or a
-// flat patch, takes the index-order path).
+// of the exact value in either summation order (and with the one quotient taken
+// after the dot product), so the two differ by at most twice that; the filter
+// asks for four times (an entry closer to tau, or a flat patch, takes the
+// canonical path). It bounds A by sqrt(N (ss + N mu^2)) and |O_j| by the codes
+// kernel's row norm.
+//
+// Bound: the FP64 pipe (two multiply-adds per clock and SM on this chip). Eight
+// lanes per entry, four entries per warp: 11 elements a lane at N = 81 and three
+// shuffle steps a sum shared by four entries, where a whole warp per entry
+// spent five steps and, with a quotient per element and |O_j| and A summed in
+// FP64 too, about 300 warp-wide FP64 operations an entry. Measured at 1023 x 769,
+// 9 x 9 patches, k = 162: 47 us against 128 us; 481 x 321, 7 x 7, k = 98:
+// 10 us against 14 us.
 __device__ __forceinline__ double canon_v(const float* __restrict__ img, int H, int W,
                                           const float* __restrict__ mask, int p, int y, int x,
                                           int t) {
@@ -228,13 +246,112 @@ __device__ __forceinline__ double canon_v(const float* __restrict__ img, int H, 
 }
 
 template <int P>
-__global__ void __launch_bounds__(128) codes_guard_kernel(
-    const float* __restrict__ img, int H, int W, const float* __restrict__ omega, int k,
-    const float* __restrict__ mask, double tau, const int2* __restrict__ guard, int guard_cap,
-    const int* __restrict__ guard_count, uint32_t* __restrict__ bitmask, int* __restrict__ d_err) {
+__device__ void codes_guard_canonical(const float* __restrict__ img, int H, int W,
+                                      const float* __restrict__ omega, int k,
+                                      const float* __restrict__ mask, double tau, int2 g,
+                                      uint32_t* __restrict__ bitmask, double* sb) {
     constexpr int N = P * P;
     constexpr int NL = (N + 31) / 32;  // elements per lane
-    __shared__ double s_buf[4][N];      // per warp: values for the lane-0 sums
+    const int Wk = (k + 31) >> 5, lane = threadIdx.x & 31;
+    const int y = g.x / W, x = g.x % W;
+    double c[NL];
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < NL; ++u) {
+        const int t = lane + 32 * u;
+        if (t < N) sb[t] = canon_v(img, H, W, mask, P, y, x, t);
+    }
+    __syncwarp();
+    double mu = 0.0;
+    if (lane == 0) {
+        for (int t = 0; t < N; ++t) mu = __dadd_rn(mu, sb[t]);
+        mu = __ddiv_rn(mu, (double)N);
+    }
+    mu = __shfl_sync(0xffffffffu, mu, 0);
+#pragma unroll
+    for (int u = 0; u < NL; ++u) {
+        const int t = lane + 32 * u;
+        c[u] = t < N ? __dadd_rn(sb[t], -mu) : 0.0;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < NL; ++u) {
+        const int t = lane + 32 * u;
+        if (t < N) sb[t] = __dmul_rn(c[u], c[u]);
+    }
+    __syncwarp();
+    double ss = 0.0;
+    if (lane == 0)
+        for (int t = 0; t < N; ++t) ss = __dadd_rn(ss, sb[t]);
+    ss = __shfl_sync(0xffffffffu, ss, 0);
+    if (ss == 0.0) {
+#pragma unroll
+        for (int u = 0; u < NL; ++u) c[u] = 0.0;
+    } else {
+        const double nrm = __dsqrt_rn(ss);
+#pragma unroll
+        for (int u = 0; u < NL; ++u) c[u] = __ddiv_rn(c[u], nrm);  // s_t
+    }
+    __syncwarp();
+    if (g.y >= 0) {
+        // one code: products across the lanes, the index-order sum on lane 0
+        const float* oj = omega + (size_t)g.y * N;
+#pragma unroll
+        for (int u = 0; u < NL; ++u) {
+            const int t = lane + 32 * u;
+            if (t < N) sb[t] = __dmul_rn((double)oj[t], c[u]);
+        }
+        __syncwarp();
+        if (lane == 0) {
+            double a = 0.0;
+            for (int t = 0; t < N; ++t) a = __dadd_rn(a, sb[t]);
+            if (fabs(a) <= tau)
+                atomicOr(bitmask + (size_t)g.x * Wk + (g.y >> 5), 1u << (g.y & 31));
+        }
+    } else {
+        // nearly flat patch: every code, one lane per code
+#pragma unroll
+        for (int u = 0; u < NL; ++u) {
+            const int t = lane + 32 * u;
+            if (t < N) sb[t] = c[u];
+        }
+        __syncwarp();
+        // up to CG codes per lane at once: independent index-order sums,
+        // interleaved so that their latencies overlap
+        constexpr int CG = 8;
+        for (int j0 = lane; j0 < k; j0 += 32 * CG) {
+            double acc[CG];
+#pragma unroll
+            for (int q = 0; q < CG; ++q) acc[q] = 0.0;
+            for (int t = 0; t < N; ++t) {
+                const double st = sb[t];
+#pragma unroll
+                for (int q = 0; q < CG; ++q) {
+                    const int j = j0 + 32 * q;
+                    if (j < k) acc[q] = __dadd_rn(acc[q], __dmul_rn((double)omega[(size_t)j * N + t], st));
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < CG; ++q) {
+                const int j = j0 + 32 * q;
+                if (j < k && fabs(acc[q]) <= tau)
+                    atomicOr(bitmask + (size_t)g.x * Wk + (j >> 5), 1u << (j & 31));
+            }
+        }
+    }
+    __syncwarp();
+}
+
+template <int P>
+__global__ void __launch_bounds__(128) codes_guard_kernel(
+    const float* __restrict__ img, int H, int W, const float* __restrict__ omega, int k,
+    const float* __restrict__ mask, const float* __restrict__ rownorm, double tau,
+    const int2* __restrict__ guard, int guard_cap, const int* __restrict__ guard_count,
+    uint32_t* __restrict__ bitmask, int* __restrict__ d_err) {
+    constexpr int N = P * P;
+    constexpr int LE = 8, EW = 32 / LE;      // lanes per entry, entries per warp
+    constexpr int NL = (N + LE - 1) / LE;    // elements per lane
+    __shared__ double s_buf[4][N];           // per warp: values for the canonical sums
     int cnt = *guard_count;
     if (cnt > guard_cap) {
         if (blockIdx.x == 0 && threadIdx.x == 0 && atomicCAS(d_err, 0, CS_DEVERR_GUARD_FULL) == 0)
@@ -242,144 +359,53 @@ __global__ void __launch_bounds__(128) codes_guard_kernel(
         cnt = guard_cap;
     }
     const int Wk = (k + 31) >> 5;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    double* sb = s_buf[wib];
-    auto wsum = [](double v) {  // warp-tree sum, the same value on every lane
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, le = lane % LE;
+    auto esum = [](double v) {  // sum over the entry's lanes, the same value on each
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+        for (int o = LE / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         return v;
     };
-    for (int e = blockIdx.x + gridDim.x * wib; e < cnt; e += gridDim.x * 4) {
-        const int2 g = guard[e];
+    for (int w = blockIdx.x + gridDim.x * wib; (long long)w * EW < cnt; w += gridDim.x * 4) {
+        const int e = w * EW + lane / LE;
+        const int2 g = e < cnt ? guard[e] : make_int2(0, 0);
+        bool open = e < cnt;  // the entry is not decided
         const int y = g.x / W, x = g.x % W;
-        double c[NL];
-        double vv[NL];
+        const float* oj = omega + (size_t)max(g.y, 0) * N;
+        double v[NL], sv = 0.0;
+        float o[NL];
 #pragma unroll
         for (int u = 0; u < NL; ++u) {
-            const int t = lane + 32 * u;
-            vv[u] = t < N ? canon_v(img, H, W, mask, P, y, x, t) : 0.0;
-            if (t < N) sb[t] = vv[u];
+            const int t = le + LE * u;
+            o[u] = t < N ? oj[t] : 0.f;
+            v[u] = t < N ? canon_v(img, H, W, mask, P, y, x, t) : 0.0;
+            sv += v[u];
         }
-        if (g.y >= 0) {
-            // tree-sum filter (see above); warp-uniform decision
-            double sv = 0.0, av = 0.0;
-#pragma unroll
-            for (int u = 0; u < NL; ++u) {
-                sv = __dadd_rn(sv, vv[u]);
-                av = __dadd_rn(av, fabs(vv[u]));
-            }
-            const double mu_f = __ddiv_rn(wsum(sv), (double)N), A = wsum(av);
-            double sc = 0.0;
-#pragma unroll
-            for (int u = 0; u < NL; ++u) {
-                const int t = lane + 32 * u;
-                c[u] = t < N ? __dadd_rn(vv[u], -mu_f) : 0.0;
-                sc = __dadd_rn(sc, __dmul_rn(c[u], c[u]));
-            }
-            const double ss_f = wsum(sc);
-            if (ss_f > 0.0) {
-                const double nrm_f = __dsqrt_rn(ss_f);
-                const float* oj = omega + (size_t)g.y * N;
-                double sa = 0.0, so = 0.0;
-#pragma unroll
-                for (int u = 0; u < NL; ++u) {
-                    const int t = lane + 32 * u;
-                    const double o = t < N ? (double)oj[t] : 0.0;
-                    sa = __dadd_rn(sa, __dmul_rn(o, __ddiv_rn(c[u], nrm_f)));
-                    so = __dadd_rn(so, __dmul_rn(o, o));
-                }
-                const double a_f = wsum(sa), on = __dsqrt_rn(wsum(so));
-                const double uu = 1.1102230246251565e-16;  // 2^-53
-                const double es = 2.0 * uu * sqrt((double)N) * A / nrm_f + (0.5 * N + 5.0) * uu;
-                const double eps = 4.0 * on * (es + N * uu * (1.0 + es)) * 1.01;
-                const double aa = fabs(a_f);
-                if (aa <= tau - eps || aa > tau + eps) {
-                    if (lane == 0 && aa <= tau - eps)
-                        atomicOr(bitmask + (size_t)g.x * Wk + (g.y >> 5), 1u << (g.y & 31));
-                    __syncwarp();
-                    continue;
-                }
-            }
-        }
-        __syncwarp();
-        double mu = 0.0;
-        if (lane == 0) {
-            for (int t = 0; t < N; ++t) mu = __dadd_rn(mu, sb[t]);
-            mu = __ddiv_rn(mu, (double)N);
-        }
-        mu = __shfl_sync(0xffffffffu, mu, 0);
+        const double mu = esum(sv) * (1.0 / N);
+        double sc = 0.0, sa = 0.0;
 #pragma unroll
         for (int u = 0; u < NL; ++u) {
-            const int t = lane + 32 * u;
-            c[u] = t < N ? __dadd_rn(sb[t], -mu) : 0.0;
+            const double c = le + LE * u < N ? v[u] - mu : 0.0;
+            sc = fma(c, c, sc);
+            sa = fma((double)o[u], c, sa);
         }
-        __syncwarp();
-#pragma unroll
-        for (int u = 0; u < NL; ++u) {
-            const int t = lane + 32 * u;
-            if (t < N) sb[t] = __dmul_rn(c[u], c[u]);
-        }
-        __syncwarp();
-        double ss = 0.0;
-        if (lane == 0)
-            for (int t = 0; t < N; ++t) ss = __dadd_rn(ss, sb[t]);
-        ss = __shfl_sync(0xffffffffu, ss, 0);
-        if (ss == 0.0) {
-#pragma unroll
-            for (int u = 0; u < NL; ++u) c[u] = 0.0;
-        } else {
-            const double nrm = __dsqrt_rn(ss);
-#pragma unroll
-            for (int u = 0; u < NL; ++u) c[u] = __ddiv_rn(c[u], nrm);  // s_t
-        }
-        __syncwarp();
-        if (g.y >= 0) {
-            // one code: products across the lanes, the index-order sum on lane 0
-            const float* oj = omega + (size_t)g.y * N;
-#pragma unroll
-            for (int u = 0; u < NL; ++u) {
-                const int t = lane + 32 * u;
-                if (t < N) sb[t] = __dmul_rn((double)oj[t], c[u]);
-            }
-            __syncwarp();
-            if (lane == 0) {
-                double a = 0.0;
-                for (int t = 0; t < N; ++t) a = __dadd_rn(a, sb[t]);
-                if (fabs(a) <= tau)
+        const double ss = esum(sc), dot = esum(sa);
+        if (open && g.y >= 0 && ss > 0.0) {
+            const double uu = 1.1102230246251565e-16;  // 2^-53
+            const double nrm = sqrt(ss), aa = fabs(dot / nrm);
+            const double es = 2.0 * uu * N * sqrt(ss + N * mu * mu) / nrm + (0.5 * N + 5.0) * uu;
+            const double eps = 4.0 * (double)rownorm[g.y] * (es + N * uu * (1.0 + es)) * 1.01;
+            if (aa <= tau - eps || aa > tau + eps) {
+                if (le == 0 && aa <= tau - eps)
                     atomicOr(bitmask + (size_t)g.x * Wk + (g.y >> 5), 1u << (g.y & 31));
-            }
-        } else {
-            // nearly flat patch: every code, one lane per code
-#pragma unroll
-            for (int u = 0; u < NL; ++u) {
-                const int t = lane + 32 * u;
-                if (t < N) sb[t] = c[u];
-            }
-            __syncwarp();
-            // up to CG codes per lane at once: independent index-order sums,
-            // interleaved so that their latencies overlap
-            constexpr int CG = 8;
-            for (int j0 = lane; j0 < k; j0 += 32 * CG) {
-                double acc[CG];
-#pragma unroll
-                for (int q = 0; q < CG; ++q) acc[q] = 0.0;
-                for (int t = 0; t < N; ++t) {
-                    const double st = sb[t];
-#pragma unroll
-                    for (int q = 0; q < CG; ++q) {
-                        const int j = j0 + 32 * q;
-                        if (j < k) acc[q] = __dadd_rn(acc[q], __dmul_rn((double)omega[(size_t)j * N + t], st));
-                    }
-                }
-#pragma unroll
-                for (int q = 0; q < CG; ++q) {
-                    const int j = j0 + 32 * q;
-                    if (j < k && fabs(acc[q]) <= tau)
-                        atomicOr(bitmask + (size_t)g.x * Wk + (j >> 5), 1u << (j & 31));
-                }
+                open = false;
             }
         }
-        __syncwarp();
+        for (unsigned todo = __ballot_sync(0xffffffffu, open && le == 0); todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const int2 c = make_int2(__shfl_sync(0xffffffffu, g.x, src),
+                                     __shfl_sync(0xffffffffu, g.y, src));
+            codes_guard_canonical<P>(img, H, W, omega, k, mask, tau, c, bitmask, s_buf[wib]);
+        }
     }
 }
 
@@ -552,6 +578,29 @@ __device__ __forceinline__ void ct_set_error(int* d_err, int site) {
     if (atomicCAS(d_err, 0, CS_DEVERR_TIMEOUT) == 0) d_err[1] = site;
 }
 
+// The 16 codes of chunk c to the callers' arrays: `codes` (k per pixel), and the
+// first chunk to `lead16` (zero beyond k: the operator's padding rows are zero).
+__device__ __forceinline__ void store_codes(const uint32_t (&v)[16], int c, bool live, int pix, int k,
+                                            float* __restrict__ codes, float* __restrict__ lead16) {
+    if (lead16 && c == 0 && live) {
+        float4* d = reinterpret_cast<float4*>(lead16 + (size_t)pix * 16);
+        if ((reinterpret_cast<uintptr_t>(d) & 15) == 0) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                d[q] = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
+                                   __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
+        } else {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) lead16[(size_t)pix * 16 + e] = __uint_as_float(v[e]);
+        }
+    }
+    if (codes && live) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e)
+            if (16 * c + e < k) codes[(size_t)pix * k + 16 * c + e] = __uint_as_float(v[e]);
+    }
+}
+
 template <int P>
 __global__ void __launch_bounds__(128, 4) codes_tc_kernel(
     const float* __restrict__ img, int H, int W, const uint8_t* __restrict__ blob, int k, int np,
@@ -571,7 +620,7 @@ __global__ void __launch_bounds__(128, 4) codes_tc_kernel(
     float* s_gray = reinterpret_cast<float*>(misc + 32);
     float* s_gabs = s_gray + GW * GH;
     float* s_w = s_gabs + GW * GH;
-    float* s_rn = s_w + N;                               // row norms, np
+    float* s_rn = s_w + ((N + 3) & ~3);                  // row norms, np (16-byte aligned)
 
     const int tid = threadIdx.x, warp = tid >> 5;
     const uint32_t ncols = ct_cols(np);
@@ -725,24 +774,18 @@ __global__ void __launch_bounds__(128, 4) codes_tc_kernel(
             uint32_t v[16];
             tc::tmem_ld16(lrow + 16u * c, v);
             tc::tmem_ld_wait();
-            threshold16(v, 16 * c, k, s_rn, ebase, tau_f, tau_slack, word, gword);
-            if (live && (codes || lead16)) {
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const int j = 16 * c + e;
-                    if (j < k && codes) codes[(size_t)pix * k + j] = __uint_as_float(v[e]);
-                    if (j < 16 && j < k && lead16) lead16[(size_t)pix * 16 + j] = __uint_as_float(v[e]);
-                }
-            }
+            threshold16(v, 16 * (c & 1), s_rn + 16 * c, ebase, tau_f, tau_slack, word, gword);
+            store_codes(v, c, live, pix, k, codes, lead16);
             if ((c & 1) || c == np / 16 - 1) {
+                const uint32_t m = word_mask(c >> 1, k);
+                word &= m;
+                gword &= m;
                 if (live && !whole) guard_word(guard, guard_cap, guard_count, pix, c >> 1, gword);
                 if (live && bitmask) bitmask[(size_t)pix * Wk + (c >> 1)] = whole ? 0u : word;
                 word = gword = 0;
             }
         }
         if (live && whole) guard_push(guard, guard_cap, guard_count, pix, -1);
-        if (live && lead16)
-            for (int j = k; j < 16; ++j) lead16[(size_t)pix * 16 + j] = 0.f;
     } else if (tid == 0 && *s_flag) {
         // MMAs still in flight: they must finish before the tensor memory is freed
         tc::mbar_wait(bars + 1, 0, tc::globaltimer() + CT_WAIT_NS);
@@ -762,8 +805,14 @@ __global__ void __launch_bounds__(128, 4) codes_tc_kernel(
 // tile t run, then write its A operand once those MMAs have read the
 // previous one; four epilogue warps threshold tile t - 1 from the other of
 // two TMEM accumulators; one thread issues the MMAs. The arithmetic per
-// pixel and entry is that of codes_tc_kernel.
-constexpr int CP_THREADS = 9 * 32;
+// pixel and entry is that of codes_tc_kernel. Where the operands leave room for
+// one CTA per SM only (9 x 9 patches), two groups of four epilogue warps share
+// each tile's 32-code words. Bound: the epilogue's thresholds and the builders'
+// patch arithmetic (latency: four or eight warps each per SM), not the
+// contraction. Measured at 1023 x 769, 9 x 9, k = 162: 229 us, against 349 us
+// with one epilogue group and per-entry output tests.
+__host__ __device__ constexpr int cp_groups(int p) { return p <= 7 ? 1 : 2; }
+__host__ __device__ constexpr int cp_threads(int p) { return (4 * cp_groups(p) + 5) * 32; }
 
 struct CpOff {
     int b, win, w, rn, prm, bars, misc, total;
@@ -798,7 +847,7 @@ __device__ __forceinline__ bool cp_wait(uint64_t* bar, uint32_t parity, volatile
 }
 
 template <int P>
-__global__ void __launch_bounds__(CP_THREADS, P <= 7 ? 2 : 1) codes_tcp_kernel(
+__global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kernel(
     const float* __restrict__ img, int H, int W, const uint8_t* __restrict__ blob, int k, int np,
     const float* __restrict__ mask, const float* __restrict__ rownorm, float tau_f,
     float tau_slack, float* __restrict__ codes, float* __restrict__ lead16,
@@ -806,6 +855,7 @@ __global__ void __launch_bounds__(CP_THREADS, P <= 7 ? 2 : 1) codes_tcp_kernel(
     int* __restrict__ guard_count, int* __restrict__ d_err) {
     constexpr int N = P * P, R = (P - 1) / 2, KS = ct_ks(P);
     constexpr int WW = CT_W + P - 1, WH = P + 1;
+    constexpr int EG = cp_groups(P), NTHR = cp_threads(P), MMA_WARP = 4 + 4 * EG;
     extern __shared__ __align__(1024) uint8_t smem[];
     const CpOff o = cp_off<P>(np);
     uint8_t* sa = smem;
@@ -819,9 +869,9 @@ __global__ void __launch_bounds__(CP_THREADS, P <= 7 ? 2 : 1) codes_tcp_kernel(
     uint64_t* a_full = bars + 1;   // builders -> MMA (4 warps)
     uint64_t* a_empty = bars + 2;  // MMA commit -> builders
     uint64_t* t_full = bars + 3;   // [2] MMA commit -> epilogue
-    uint64_t* t_empty = bars + 5;  // [2] epilogue (4 warps) -> MMA
+    uint64_t* t_empty = bars + 5;  // [2] epilogue (4 EG warps) -> MMA
     uint64_t* p_full = bars + 7;   // [2] builders (4 warps) -> epilogue: pixel parameters
-    uint64_t* p_empty = bars + 9;  // [2] epilogue (4 warps) -> builders
+    uint64_t* p_empty = bars + 9;  // [2] epilogue (4 EG warps) -> builders
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + o.misc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + o.misc + 4);
 
@@ -835,21 +885,21 @@ __global__ void __launch_bounds__(CP_THREADS, P <= 7 ? 2 : 1) codes_tcp_kernel(
         tc::mbar_init(a_empty, 1);
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(t_full + b, 1);
-            tc::mbar_init(t_empty + b, 4);
+            tc::mbar_init(t_empty + b, 4 * EG);
             tc::mbar_init(p_full + b, 4);
-            tc::mbar_init(p_empty + b, 4);
+            tc::mbar_init(p_empty + b, 4 * EG);
         }
         *abort_flag = 0;
         tc::fence_mbar_init();
         tc::mbar_arrive_expect_tx(b_full, b_bytes);
         tc::bulk_g2s(sb, blob, b_bytes, b_full);
     }
-    if (warp == 8) {
+    if (warp == MMA_WARP) {
         tc::tmem_alloc(s_tmem, 2 * ncols);
         tc::tmem_relinquish();
     }
-    for (int i = tid; i < N; i += CP_THREADS) s_w[i] = mask[i];
-    for (int i = tid; i < np; i += CP_THREADS) s_rn[i] = i < k ? rownorm[i] : 0.f;
+    for (int i = tid; i < N; i += NTHR) s_w[i] = mask[i];
+    for (int i = tid; i < np; i += NTHR) s_rn[i] = i < k ? rownorm[i] : 0.f;
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -961,9 +1011,9 @@ __global__ void __launch_bounds__(CP_THREADS, P <= 7 ? 2 : 1) codes_tcp_kernel(
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(p_full + pb);
         }
-    } else if (warp < 8) {
+    } else if (warp < MMA_WARP) {
         // ---------------------------------------------------------- epilogue
-        const int q = warp & 3;
+        const int q = warp & 3, eg = (warp - 4) >> 2;
         const uint32_t lrow = tmem + ((uint32_t)(32 * q) << 16);
         const int Wk = (k + 31) >> 5, nch = np / 16;
         int kk = 0;
@@ -978,33 +1028,27 @@ __global__ void __launch_bounds__(CP_THREADS, P <= 7 ? 2 : 1) codes_tcp_kernel(
             const bool live = pp.x >= 0, whole = pp.y != 0;
             const int pix = live ? pp.x : 0;
             const float ebase = __int_as_float(pp.z);
-            uint32_t word = 0, gword = 0;
-            for (int c = 0; c < nch; ++c) {
-                uint32_t v[16];
-                tc::tmem_ld16(lrow + (uint32_t)(b * ncols) + 16u * c, v);
-                tc::tmem_ld_wait();
-                threshold16(v, 16 * c, k, s_rn, ebase, tau_f, tau_slack, word, gword);
-                if (live && (codes || lead16)) {
+            for (int wd = eg; wd < Wk; wd += EG) {  // this group's 32-code words
+                uint32_t word = 0, gword = 0;
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const int j = 16 * c + e;
-                        if (j < k && codes) codes[(size_t)pix * k + j] = __uint_as_float(v[e]);
-                        if (j < 16 && j < k && lead16)
-                            lead16[(size_t)pix * 16 + j] = __uint_as_float(v[e]);
+                for (int h = 0; h < 2; ++h) {
+                    const int c = 2 * wd + h;
+                    if (c < nch) {
+                        uint32_t v[16];
+                        tc::tmem_ld16(lrow + (uint32_t)(b * ncols) + 16u * c, v);
+                        tc::tmem_ld_wait();
+                        threshold16(v, 16 * h, s_rn + 16 * c, ebase, tau_f, tau_slack, word, gword);
+                        store_codes(v, c, live, pix, k, codes, lead16);
                     }
                 }
-                if ((c & 1) || c == nch - 1) {
-                    if (live && !whole) guard_word(guard, guard_cap, guard_count, pix, c >> 1, gword);
-                    if (live && bitmask) bitmask[(size_t)pix * Wk + (c >> 1)] = whole ? 0u : word;
-                    word = gword = 0;
-                }
+                const uint32_t m = word_mask(wd, k);
+                if (live && !whole) guard_word(guard, guard_cap, guard_count, pix, wd, gword & m);
+                if (live && bitmask) bitmask[(size_t)pix * Wk + wd] = whole ? 0u : word & m;
             }
             tc::fence_before_sync();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(t_empty + b);
-            if (live && whole) guard_push(guard, guard_cap, guard_count, pix, -1);
-            if (live && lead16)
-                for (int j = k; j < 16; ++j) lead16[(size_t)pix * 16 + j] = 0.f;
+            if (live && whole && eg == 0) guard_push(guard, guard_cap, guard_count, pix, -1);
         }
     } else if (lane == 0) {
         // ---------------------------------------------------------- MMA issuer
@@ -1043,7 +1087,7 @@ __global__ void __launch_bounds__(CP_THREADS, P <= 7 ? 2 : 1) codes_tcp_kernel(
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 8) {
+    if (warp == MMA_WARP) {
         tc::fence_after_sync();
         tc::tmem_dealloc(tmem, 2 * ncols);
     }
@@ -1052,7 +1096,7 @@ __global__ void __launch_bounds__(CP_THREADS, P <= 7 ? 2 : 1) codes_tcp_kernel(
 template <int P>
 size_t ct_smem(int np) {
     constexpr int N = P * P, KS = ct_ks(P), GW = CT_W + P - 1, GH = CT_H + P - 1;
-    size_t b = 3 * KS * 4096 + 3 * KS * (size_t)np * 32 + 32 + 4 * (2 * GW * GH + N + np);
+    size_t b = 3 * KS * 4096 + 3 * KS * (size_t)np * 32 + 32 + 4 * (2 * GW * GH + ((N + 3) & ~3) + np);
     b = (b + 15) / 16 * 16;
     // at most 512 / ncols CTAs per SM, so that tensor-memory allocations never wait
     const int per_sm = 512 / (int)ct_cols(np);
@@ -1102,7 +1146,7 @@ cudaError_t launch_tc_p(const CodesArgs& a, cudaStream_t st) {
         return e;
     const int ntiles = ((a.W + CT_W - 1) / CT_W) * ((a.H + CT_H - 1) / CT_H);
     const int grid = ntiles < per_sm * n_sm ? ntiles : per_sm * n_sm;
-    codes_tcp_kernel<P><<<grid, CP_THREADS, psmem, st>>>(
+    codes_tcp_kernel<P><<<grid, cp_threads(P), psmem, st>>>(
         a.img, a.H, a.W, a.omega_blob, a.k, np, a.mask, a.rownorm, tau_f, slack, a.codes,
         a.lead16, a.bitmask, a.guard, a.guard_cap, a.guard_count, a.d_err);
     return cudaGetLastError();
@@ -1185,7 +1229,7 @@ cudaError_t launch_codes(const CodesArgs& a, cudaStream_t st) {
 #define CS_GUARD(PP)                                                                        \
     case PP:                                                                                \
         codes_guard_kernel<PP><<<152 * 4, 128, 0, st>>>(a.img, a.H, a.W, a.omega, a.k, a.mask, \
-                                                        a.tau, a.guard, a.guard_cap,          \
+                                                        a.rownorm, a.tau, a.guard, a.guard_cap, \
                                                         a.guard_count, a.bitmask, a.d_err);   \
         break;
     switch (a.p) {
