@@ -594,7 +594,6 @@ void cs_lik_carve(Carve& c, LikPlan& L, int32_t* dist2) {
     L.t.sg = c.take<float>(S);
     L.t.sb = c.take<float>(S);
     L.t.sbits = c.take<uint32_t>((size_t)Wk * S);
-    L.t.spop = c.take<int32_t>(S);
     L.t.rep = c.take<uint32_t>((size_t)n * Wk);
     L.t.blob = c.take<uint8_t>((size_t)L.total_tiles * L.stage_bytes, 1024);
     L.t.tile_xy = c.take<uint32_t>(L.tc_form ? (size_t)L.total_tiles * tc_tile_samples() : 0);
@@ -698,8 +697,8 @@ TcLaunch cs_tc_launch(cs_ctx* ctx, const LikPlan& L, const float* img, const uin
     return T;
 }
 
-// Gather and sum; with `sorted` the tensor-core sample order was already
-// enqueued (cs_data_term sorts on a side stream). The gather and the
+// Sample tiles and sum; with `sorted` the tensor-core sample order was already
+// enqueued (cs_data_term sorts on a side stream). The majority co-supports and the
 // tensor-core tile build do not need the distances: with `dist_ready` (the
 // distance transform's completion on another stream) the stream waits for
 // it only before the sum itself.
@@ -718,13 +717,12 @@ static cudaError_t enqueue_sum(cs_ctx* ctx, const LikPlan& L, const float* img,
     cudaError_t e;
     {
         StageTimer tm(ctx, CS_STAGE_GATHER, st);
+        e = L.tc_form ? launch_sum_tc_prepare(T, sorted, st)
+                      : launch_plain_tiles(img, L.H, L.W, bitmask, L.k, L.n_labels, L.d_off,
+                                           sample_pix, L.total_tiles, L.persample, L.t.blob, st);
         // (the smooth texture has representatives of its own)
-        e = launch_gather(img, L.H, L.W, bitmask, L.k, L.n_labels, L.d_off, sample_pix, L.S,
-                          prm->mode == CS_MODE_FACTORISED, L.t, st);
-        if (e == cudaSuccess)
-            e = L.tc_form ? launch_sum_tc_prepare(T, sorted, st)
-                          : launch_plain_tiles(L.d_off, L.n_labels, L.total_tiles, L.k, L.S,
-                                               L.persample, L.t, st);
+        if (e == cudaSuccess && prm->mode == CS_MODE_FACTORISED)
+            e = launch_majority(L.H, L.W, bitmask, L.k, L.n_labels, L.d_off, sample_pix, L.t.rep, st);
     }
     if (e == cudaSuccess && dist_ready) e = cudaStreamWaitEvent(st, dist_ready, 0);
     if (e != cudaSuccess) return e;
@@ -811,17 +809,18 @@ cs_status cs_plan_likelihood(cs_ctx* ctx, LikPlan& L, int H, int W, int k, int n
     return CS_OK;
 }
 
-// distances, sample tables and the plain form's sample tiles
+// distances, majority co-supports and the plain form's sample tiles
 cudaError_t cs_enqueue_prepare(cs_ctx* ctx, const LikPlan& L, const float* img,
                                const uint32_t* bitmask, const int32_t* sample_pix,
                                const cs_params* prm, cudaStream_t st) {
     cudaError_t e = enqueue_distances(ctx, L, sample_pix, st);
     if (e != cudaSuccess) return e;
     StageTimer tm(ctx, CS_STAGE_GATHER, st);
-    e = launch_gather(img, L.H, L.W, bitmask, L.k, L.n_labels, L.d_off, sample_pix, L.S,
-                      prm->mode == CS_MODE_FACTORISED, L.t, st);
+    if (prm->mode == CS_MODE_FACTORISED)
+        e = launch_majority(L.H, L.W, bitmask, L.k, L.n_labels, L.d_off, sample_pix, L.t.rep, st);
     if (e != cudaSuccess || L.tc_form) return e;
-    return launch_plain_tiles(L.d_off, L.n_labels, L.total_tiles, L.k, L.S, L.persample, L.t, st);
+    return launch_plain_tiles(img, L.H, L.W, bitmask, L.k, L.n_labels, L.d_off, sample_pix,
+                              L.total_tiles, L.persample, L.t.blob, st);
 }
 
 // exact plain sum over a device pixel list (after cs_enqueue_prepare): with

@@ -159,9 +159,9 @@ static cudaError_t enqueue_run(cs_batch* b, cudaStream_t st) {
             e = launch_edt(ea, ss);
         }
         if (e == cudaSuccess && !b->codes_given) e = launch_codes(m.codes, ss);
-        if (e == cudaSuccess)
-            e = launch_gather(m.d.img, L.H, L.W, m.codes.bitmask, L.k, L.n_labels, L.d_off,
-                              m.d.sample_pix, L.S, !L.persample, L.t, ss);
+        if (e == cudaSuccess && b->prm.mode == CS_MODE_FACTORISED)
+            e = launch_majority(L.H, L.W, m.codes.bitmask, L.k, L.n_labels, L.d_off, m.d.sample_pix,
+                                L.t.rep, ss);
         if (e != cudaSuccess) break;
         if (b->tc) {
             TcLaunch T = cs_tc_launch(ctx, L, m.d.img, m.codes.bitmask, m.d.sample_pix, &b->prm,
@@ -172,7 +172,8 @@ static cudaError_t enqueue_run(cs_batch* b, cudaStream_t st) {
             T.first_ptile = b->first_ptile[s];
             e = launch_tc_prepare(T, ss);
         } else {
-            e = launch_plain_tiles(L.d_off, L.n_labels, L.total_tiles, L.k, L.S, L.persample, L.t, ss);
+            e = launch_plain_tiles(m.d.img, L.H, L.W, m.codes.bitmask, L.k, L.n_labels, L.d_off,
+                                   m.d.sample_pix, L.total_tiles, L.persample, L.t.blob, ss);
             if (e == cudaSuccess)
                 e = launch_sum_plain(cs_sum_args(ctx, L, m.d.img, m.codes.bitmask, &b->prm,
                                                  m.d.neglog, m.d.post), ss);

@@ -260,7 +260,8 @@ struct OffsetsParam {
 };
 cudaError_t launch_set_offsets(const OffsetsParam& p, int n, int32_t* dst, cudaStream_t st);
 
-// Per-sample tables (SoA) and the majority co-support of each label.
+// Per-sample tables (SoA; tensor-core forms, written with their tiles) and the
+// majority co-support of each label.
 struct SampleTables {
     float* sx;
     float* sy;
@@ -268,15 +269,14 @@ struct SampleTables {
     float* sg;
     float* sb;
     uint32_t* sbits;  // word-major: [Wk][S]
-    int32_t* spop;    // popcount of each sample's bitmask
     uint32_t* rep;    // [n_labels][Wk]
     uint8_t* blob;    // sample tiles (tensor-core form: ring-stage layout)
     uint32_t* tile_xy;  // tensor-core tile slots: sample position x | y << 16
     int32_t* perm;    // tensor-core sample order (Morton order in chunks of 4096)
 };
-cudaError_t launch_gather(const float* img, int H, int W, const uint32_t* bitmask, int k,
-                          int n_labels, const int32_t* d_label_off, const int32_t* sample_pix,
-                          int n_samples, bool want_rep, const SampleTables& t, cudaStream_t st);
+cudaError_t launch_majority(int H, int W, const uint32_t* bitmask, int k, int n_labels,
+                            const int32_t* d_label_off, const int32_t* sample_pix, uint32_t* rep,
+                            cudaStream_t st);
 
 // Pixel x sample likelihood sum and label normalisation.
 struct SumArgs {
@@ -308,9 +308,10 @@ struct SumArgs {
 cudaError_t launch_sum_plain(const SumArgs& a, cudaStream_t st);
 int plain_tiles_per_label(int m);
 size_t plain_tile_bytes(int k, bool persample);
-cudaError_t launch_plain_tiles(const int32_t* d_label_off, int n_labels, int total_tiles, int k,
-                               int n_samples, bool persample, const SampleTables& t,
-                               cudaStream_t st);
+cudaError_t launch_plain_tiles(const float* img, int H, int W, const uint32_t* bitmask, int k,
+                               int n_labels, const int32_t* d_label_off,
+                               const int32_t* sample_pix, int total_tiles, bool persample,
+                               uint8_t* blob, cudaStream_t st);
 
 struct TcImage;
 
@@ -452,7 +453,7 @@ int tc_tile_samples();  // samples per tensor-core sample tile
 int tc_pixel_tiles(int H, int W);
 bool tc_supported(int k, bool tex8);
 // Morton order of the samples (needs only the label offsets and sample
-// pixels), then the sample tiles (needs the gathered tables; writes *L.desc),
+// pixels), then the sample tiles (needs the sample order; writes *L.desc),
 // or both.
 cudaError_t launch_tc_sort(const TcLaunch& L, cudaStream_t st);
 cudaError_t launch_tc_tiles(const TcLaunch& L, cudaStream_t st);
@@ -466,7 +467,7 @@ cudaError_t launch_tc_sum(const TcImage* descs, int n_images, const TcSumParams&
                           cudaStream_t st);
 // For a single image (L.desc must be set): the preparation (Morton sort and
 // tile build, or the tile build alone when `sorted`), which needs the
-// gathered sample tables but not the distances, then the sum.
+// bitmasks but not the distances, then the sum.
 cudaError_t launch_sum_tc_prepare(const TcLaunch& L, bool sorted, cudaStream_t st);
 cudaError_t launch_sum_tc_run(const TcLaunch& L, cudaStream_t st);
 

@@ -7,17 +7,15 @@
 //   2. row pass (one warp per label and row): horizontal distance h to the
 //      nearest seed in the same row, from bit scans of the bitmap words;
 //   3. column pass (2, 4 or 8 builder threads per label and column, one per
-//      row segment, and eight readers): lower envelopes of the parabolas
+//      row segment, and 32 readers): lower envelopes of the parabolas
 //      (y - q)^2 + h(q)^2 over each segment's rows q with finite h, each
 //      built in one sweep and read back by row ranges; intersection
 //      abscissae are compared as exact rationals with 64-bit cross products,
 //      so the result equals the brute-force minimum bit for bit. For images
-//      with few columns and rows (labels x width < 16384, height <= 64) an
-//      outward scan per pixel with early exit gives the same minimum with
-//      far more parallelism.
-// The sample gather builds SoA tables of every sample (location, colour,
-// co-support bitmask and its popcount) and, for the factorised form, the
-// majority co-support of each label (Eq. tex-rep: bit set iff 2 * count >= m).
+//      up to labels x width x height^2 = 2e7 an outward scan per pixel with early
+//      exit gives the same minimum with far more parallelism.
+// majority_kernel: for the factorised form, the majority co-support of each label
+// (Eq. tex-rep: bit set iff 2 * count >= m).
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
@@ -89,19 +87,23 @@ __global__ void rows_binary_kernel(int H, int W, int n_labels, const uint32_t* _
     }
 }
 
-// Column pass, split: in each block of 32 columns S warps build the lower
-// envelopes of every column, warp b over the rows of segment b (one thread
-// per column and segment; one sweep over the segment's rows with finite h: a
-// row's parabola (y - q)^2 + h(q)^2 replaces the stack top while it lies
-// below it from the top's breakpoint on, compared exactly with 64-bit cross
-// products); then all NSEG warps read them back, warp s for the rows
-// [s H / NSEG, (s + 1) H / NSEG): each thread finds the segment of its first
-// row in each of the S envelopes by binary search over the breakpoints (the
-// same exact comparison, monotone in the segment index), walks on, and keeps
-// the smallest of the S values, the minimum over all rows. More segments
-// shorten the sequential sweeps at the cost of more envelopes per read.
-constexpr int NSEG = 8;  // reader warps per block (and the most segments)
-
+// Column pass, split: a block of 256 threads takes CB columns. S threads per
+// column build the lower envelopes of its S row segments (one sweep over the
+// segment's rows with finite h: a row's parabola (y - q)^2 + h(q)^2 replaces the
+// stack top while it lies below it from the top's breakpoint on, compared exactly
+// with 64-bit cross products); then NRD threads per column read them back, each
+// for a range of rows: it finds the segment of its first row in each of the S
+// envelopes by binary search over the breakpoints (the same exact comparison,
+// monotone in the segment index), walks on, and keeps the smallest of the S
+// values, the minimum over all rows.
+//
+// Bound: the sweeps' and the reads' latency: about 0.2 us a row swept and 0.13 us
+// a row and envelope read. Few columns per block give many readers (H / 32 rows
+// each) and blocks for every SM, and with them more segments pay. Measured at
+// 481 x 321, 5 labels: 28 us, against 42 us with 32 columns per block, 4
+// segments and 8 readers (and 54 us with 8 segments).
+constexpr int CB = 8;          // columns per block
+constexpr int NRD = 256 / CB;  // reader threads per column
 
 __device__ __forceinline__ int env_build(const int32_t* __restrict__ col, int W, int q_lo, int q_hi,
                                          int32_t* v, int32_t* F, long long stride) {
@@ -167,15 +169,15 @@ __device__ __forceinline__ int32_t env_value(EnvCursor& c, const int32_t* v, con
 }
 
 template <bool SHARED, int S>
-__global__ void __launch_bounds__(32 * NSEG) cols_envelope_split_kernel(
+__global__ void __launch_bounds__(256) cols_envelope_split_kernel(
     int H, int W, int n_labels, const int32_t* __restrict__ h, int32_t* __restrict__ gv,
     int32_t* __restrict__ gF, int32_t* __restrict__ dist2) {
-    static_assert(S >= 1 && S <= NSEG, "segments");
+    static_assert(S >= 1 && S <= NRD, "segments");
     extern __shared__ int32_t smem[];
-    __shared__ int s_kk[S][32];
+    __shared__ int s_kk[S][CB];
     const long long ncol = (long long)n_labels * W;
-    const int c = threadIdx.x & 31, seg = threadIdx.x >> 5;
-    const long long col_id = blockIdx.x * 32ll + c;
+    const int c = threadIdx.x % CB, seg = threadIdx.x / CB;
+    const long long col_id = blockIdx.x * (long long)CB + c;
     const bool valid = col_id < ncol;
     const int i = valid ? (int)(col_id / W) : 0, x = valid ? (int)(col_id % W) : 0;
     const int HS = (H + S - 1) / S;  // rows (and stack entries) per segment
@@ -183,8 +185,8 @@ __global__ void __launch_bounds__(32 * NSEG) cols_envelope_split_kernel(
     long long stride;
     if (SHARED) {
         v = smem + c;
-        F = smem + (size_t)S * HS * 32 + c;
-        stride = 32;
+        F = smem + (size_t)S * HS * CB + c;
+        stride = CB;
     } else {
         v = gv + col_id;
         F = gF + col_id;
@@ -200,13 +202,13 @@ __global__ void __launch_bounds__(32 * NSEG) cols_envelope_split_kernel(
     __syncthreads();  // envelopes complete (shared or global) for the whole block
     if (!valid) return;
     int32_t* out = dist2 + (size_t)i * H * W + x;
-    const int y0 = (int)((long long)H * seg / NSEG), y1 = (int)((long long)H * (seg + 1) / NSEG);
+    const int y0 = (int)((long long)H * seg / NRD), y1 = (int)((long long)H * (seg + 1) / NRD);
     EnvCursor cur[S];
     int kk[S];
 #pragma unroll
     for (int b = 0; b < S; ++b) {
         kk[b] = s_kk[b][c];
-        if (kk[b] >= 0)
+        if (kk[b] >= 0 && y0 < y1)
             cur[b] = env_seek(v + (size_t)b * HS * stride, F + (size_t)b * HS * stride, stride,
                               kk[b], y0);
     }
@@ -221,59 +223,50 @@ __global__ void __launch_bounds__(32 * NSEG) cols_envelope_split_kernel(
     }
 }
 
-// Column pass for small images (one thread per label and pixel, x fastest):
-// D(y) = min over rows q of h(q)^2 + (y - q)^2, scanning q outwards from y
-// and stopping once (y - q)^2 alone reaches the best value found, which no
-// farther row can beat. Exact (integer arithmetic); O(min(H, sqrt(D))) per
-// pixel, so it is chosen only for short images whose envelope pass has too
-// few columns to fill the GPU.
-__global__ void cols_scan_kernel(int H, int W, int n_labels, const int32_t* __restrict__ h,
-                                 int32_t* __restrict__ dist2) {
-    const long long P = (long long)H * W;
-    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (tid >= P * n_labels) return;
-    const int i = (int)(tid / P);
-    const int rem = (int)(tid % P), y = rem / W, x = rem % W;
-    const int32_t* col = h + (size_t)i * P + x;
-    const int32_t h0 = col[(size_t)y * W];
-    int32_t D = h0 == INF ? INF : h0 * h0;
-    for (int d = 1; d < H; ++d) {
-        const int32_t d2 = d * d;
-        if (d2 >= D) break;
-        const bool up = y >= d, dn = y + d < H;
-        if (!up && !dn) break;
-        if (up) {
-            const int32_t a = col[(size_t)(y - d) * W];
-            if (a != INF) D = min(D, a * a + d2);
-        }
-        if (dn) {
-            const int32_t b = col[(size_t)(y + d) * W];
-            if (b != INF) D = min(D, b * b + d2);
-        }
+// Column pass for small images: D(y) = min over rows q of h(q)^2 + (y - q)^2,
+// scanning q outwards from y and stopping once (y - q)^2 alone reaches the best
+// value found, which no farther row can beat. Exact (integer arithmetic). A
+// block holds 32 columns' h^2 in shared memory and scans `rows` rows of them,
+// one row per warp at a time, SCAN_D rows each way per step. (Past the image's
+// edge the edge row's h^2 is taken again with the larger distance: a value that
+// the edge row itself has beaten.) O(min(H, sqrt(D))) per pixel with full
+// parallelism, where the envelopes' sequential sweeps leave most of the chip
+// idle (at 481 x 321, 5 labels the scan takes about 110 us: the distances are
+// long). Measured at 96 x 64, 3 labels: 5.2 us against 17 us of a scan in global
+// memory, one row per step.
+constexpr int SCAN_D = 4;
+constexpr int32_t SCAN_INF = 0x40000000;  // + any (y - q)^2 stays below 2^31
+__global__ void __launch_bounds__(256) cols_scan_kernel(int H, int W, int n_labels, int rows,
+                                                        const int32_t* __restrict__ h,
+                                                        int32_t* __restrict__ dist2) {
+    extern __shared__ int32_t hh[];  // H x 32
+    const long long ncol = (long long)n_labels * W;
+    const int c = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long col_id = blockIdx.x * 32ll + c;
+    const bool valid = col_id < ncol;
+    const int i = valid ? (int)(col_id / W) : 0, x = valid ? (int)(col_id % W) : 0;
+    const size_t base = (size_t)i * H * W + x;
+    for (int q = warp; q < H; q += 8) {
+        const int32_t v = valid ? h[base + (size_t)q * W] : INF;
+        hh[q * 32 + c] = v == INF ? SCAN_INF : v * v;
     }
-    dist2[(size_t)i * P + rem] = D;
-}
-
-__global__ void gather_kernel(const float* __restrict__ img, int W, long long P,
-                              const uint32_t* __restrict__ bitmask, int Wk,
-                              const int32_t* __restrict__ sample_pix, int n_samples,
-                              SampleTables t) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n_samples) return;
-    int pix = sample_pix[s];
-    if (pix < 0 || pix >= P) pix = 0;  // reported by seed_kernel; keep the tables finite
-    t.sx[s] = (float)(pix % W);
-    t.sy[s] = (float)(pix / W);
-    t.sr[s] = img[(size_t)pix * 3 + 0];
-    t.sg[s] = img[(size_t)pix * 3 + 1];
-    t.sb[s] = img[(size_t)pix * 3 + 2];
-    int pc = 0;
-    for (int w = 0; w < Wk; ++w) {
-        uint32_t b = bitmask[(size_t)pix * Wk + w];
-        t.sbits[(size_t)w * n_samples + s] = b;
-        pc += __popc(b);
+    __syncthreads();
+    const int y1 = min(H, ((int)blockIdx.y + 1) * rows);
+    for (int y = blockIdx.y * rows + warp; y < y1; y += 8) {
+        int32_t D = hh[y * 32 + c];
+        const int reach = max(y, H - 1 - y);
+        for (int d = 1; d <= reach && d * d < D; d += SCAN_D) {
+            int32_t m = SCAN_INF;
+#pragma unroll
+            for (int r = 0; r < SCAN_D; ++r) {
+                const int e = d + r;
+                const int32_t up = hh[max(y - e, 0) * 32 + c], dn = hh[min(y + e, H - 1) * 32 + c];
+                m = min(m, min(up, dn) + e * e);
+            }
+            D = min(D, m);
+        }
+        if (valid) dist2[base + (size_t)y * W] = D >= SCAN_INF ? INF : D;
     }
-    t.spop[s] = pc;
 }
 
 // Majority co-support of a label, one block per (word, label): each warp
@@ -281,17 +274,23 @@ __global__ void gather_kernel(const float* __restrict__ img, int W, long long P,
 // bit b of all of them, and adds its population count. Bound: latency.
 // Measured at 4 labels of up to 3100 samples, k = 98: 7 us, against 100 us
 // with one thread per (label, bit) walking the samples.
-constexpr int MJ = 256;
+constexpr int MJ = 1024;
 __global__ void __launch_bounds__(MJ) majority_kernel(const int32_t* __restrict__ off, int k,
-                                                      int Wk, int n_samples,
-                                                      const uint32_t* __restrict__ sbits,
+                                                      int Wk, long long P,
+                                                      const int32_t* __restrict__ sample_pix,
+                                                      const uint32_t* __restrict__ bitmask,
                                                       uint32_t* __restrict__ rep) {
     __shared__ int s_cnt[MJ / 32][32];
     const int w = blockIdx.x, i = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int s0 = off[i], s1 = off[i + 1];
     int cnt = 0;
     for (int s = s0 + 32 * warp; s < s1; s += MJ) {
-        uint32_t v = s + lane < s1 ? sbits[(size_t)w * n_samples + s + lane] : 0u;
+        uint32_t v = 0u;
+        if (s + lane < s1) {
+            int pix = sample_pix[s + lane];
+            if (pix < 0 || pix >= P) pix = 0;  // reported by seed_kernel
+            v = bitmask[(size_t)pix * Wk + w];
+        }
         uint32_t m = 0x0000FFFFu;
 #pragma unroll
         for (int j = 16; j > 0; j >>= 1, m ^= m << j) {
@@ -330,48 +329,57 @@ cudaError_t launch_edt(const EdtArgs& a, cudaStream_t st) {
     rows_binary_kernel<<<(unsigned)((nrow * 32 + 127) / 128), 128, 0, st>>>(
         a.H, a.W, a.n_labels, a.seedbits, a.colbuf);
     const long long ncol = (long long)a.n_labels * a.W;
-    if (ncol < 16384 && a.H <= 64) {
-        // too few columns for the envelope pass to fill the GPU: scan per pixel
-        const long long n = (long long)a.n_labels * a.H * a.W;
-        cols_scan_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a.H, a.W, a.n_labels,
-                                                                       a.colbuf, a.dist2);
+    // the scan's work is at most about ncol H^2 / 1.5 row visits (all of them when
+    // the distances exceed the height): up to SCAN_MOST it stays below the
+    // envelopes' time (at 240 x 160, 8 labels, 4.9e7, the two are equal); a column
+    // block's h^2 must fit shared memory (H <= 880)
+    constexpr long long SCAN_MOST = 20000000ll;
+    if (ncol * a.H * a.H <= SCAN_MOST && a.H <= 880) {
+        const unsigned cb = (unsigned)((ncol + 31) / 32);
+        // rows per block: about two blocks per SM, a multiple of the 8 warps
+        int rows = (int)std::min<long long>(64, std::max<long long>(8, (long long)cb * a.H / 304));
+        rows = (rows + 7) / 8 * 8;
+        cudaError_t e2 = cudaFuncSetAttribute(cols_scan_kernel,
+                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              880 * 128);
+        if (e2 != cudaSuccess) return e2;
+        cols_scan_kernel<<<dim3(cb, (a.H + rows - 1) / rows), 256, (size_t)a.H * 128, st>>>(
+            a.H, a.W, a.n_labels, rows, a.colbuf, a.dist2);
         return cudaGetLastError();
     }
-    // envelopes of 32 columns per block (S segments) in shared memory when they fit
-    const unsigned nblk = (unsigned)((ncol + 31) / 32);
+    // envelopes of CB columns per block (S segments) in shared memory when they fit
+    const unsigned nblk = (unsigned)((ncol + CB - 1) / CB);
     auto run = [&](auto seg_c) -> cudaError_t {
         constexpr int S = decltype(seg_c)::value;
-        const size_t smem = (size_t)((a.H + S - 1) / S) * S * 2 * sizeof(int32_t) * 32;
+        const size_t smem = (size_t)((a.H + S - 1) / S) * S * 2 * sizeof(int32_t) * CB;
         if (smem <= 110u * 1024u) {
+            // (the limit of every size: captured launches of several sizes share it)
             cudaError_t e2 = cudaFuncSetAttribute(cols_envelope_split_kernel<true, S>,
                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)smem);
+                                                  110 * 1024);
             if (e2 != cudaSuccess) return e2;
-            cols_envelope_split_kernel<true, S><<<nblk, 32 * NSEG, smem, st>>>(
+            cols_envelope_split_kernel<true, S><<<nblk, 256, smem, st>>>(
                 a.H, a.W, a.n_labels, a.colbuf, nullptr, nullptr, a.dist2);
         } else {
-            cols_envelope_split_kernel<false, S><<<nblk, 32 * NSEG, 0, st>>>(
+            cols_envelope_split_kernel<false, S><<<nblk, 256, 0, st>>>(
                 a.H, a.W, a.n_labels, a.colbuf, a.vbuf, a.fbuf, a.dist2);
         }
         return cudaSuccess;
     };
-    // the fewest segments (2, 4 or 8) whose sweeps are at most 128 rows long
-    e = a.H > 512 ? run(std::integral_constant<int, 8>{})
-      : a.H > 256 ? run(std::integral_constant<int, 4>{})
-                  : run(std::integral_constant<int, 2>{});
+    // sweeps and reads balance at about 7 segments of H rows; short images have
+    // too few rows for as many
+    e = a.H > 64 ? run(std::integral_constant<int, 8>{})
+      : a.H > 32 ? run(std::integral_constant<int, 4>{})
+                 : run(std::integral_constant<int, 2>{});
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
-cudaError_t launch_gather(const float* img, int H, int W, const uint32_t* bitmask, int k,
-                          int n_labels, const int32_t* d_label_off, const int32_t* sample_pix,
-                          int n_samples, bool want_rep, const SampleTables& t, cudaStream_t st) {
+cudaError_t launch_majority(int H, int W, const uint32_t* bitmask, int k, int n_labels,
+                            const int32_t* d_label_off, const int32_t* sample_pix, uint32_t* rep,
+                            cudaStream_t st) {
     const int Wk = (k + 31) / 32;
-    gather_kernel<<<(n_samples + 255) / 256, 256, 0, st>>>(img, W, (long long)H * W, bitmask, Wk, sample_pix,
-                                                           n_samples, t);
-    if (want_rep) {
-        majority_kernel<<<dim3(Wk, n_labels), MJ, 0, st>>>(d_label_off, k, Wk, n_samples,
-                                                           t.sbits, t.rep);
-    }
+    majority_kernel<<<dim3(Wk, n_labels), MJ, 0, st>>>(d_label_off, k, Wk, (long long)H * W,
+                                                       sample_pix, bitmask, rep);
     return cudaGetLastError();
 }

@@ -122,10 +122,7 @@ __device__ __forceinline__ void label_consts(int D, float alpha, float d_min, fl
 
 // The four bytes of a nibble's codes: `one` where the bit is set, else 0.
 __device__ __forceinline__ uint32_t spread(uint32_t nibble, uint32_t one) {
-    uint32_t w = 0;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) w |= ((nibble >> e) & 1u ? one : 0u) << (8 * e);
-    return w;
+    return (nibble * 0x00204081u & 0x01010101u) * one;
 }
 constexpr uint32_t E4M3_ONE = 0x38u, E4M3_MINUS = 0xB8u;
 // e4m3 of -v, v an integer below 16 times a power of two (four significant bits: exact)
@@ -138,8 +135,10 @@ __device__ __forceinline__ uint32_t e4m3_minus(int v) {
 // Sample tiles: one thread per (tile, sample). Padded samples lie far away (their
 // terms vanish) and have no codes.
 __global__ void __launch_bounds__(256) plain_tiles_kernel(
+    const float* __restrict__ img, int W, long long P, const uint32_t* __restrict__ bitmask, int Wk,
     const int32_t* __restrict__ label_off, const int32_t* __restrict__ tile_off, int n_labels,
-    int total_tiles, SampleTables t, int n_samples, int k, int KS, uint8_t* __restrict__ blob) {
+    const int32_t* __restrict__ sample_pix, int total_tiles, int k, int KS,
+    uint8_t* __restrict__ blob) {
     const long long gid = blockIdx.x * 256ll + threadIdx.x;
     if (gid >= (long long)total_tiles * TS) return;
     const int tile = (int)(gid / TS), r = (int)(gid % TS);
@@ -152,13 +151,14 @@ __global__ void __launch_bounds__(256) plain_tiles_kernel(
     const bool ok = s < label_off[lo + 1];
     uint8_t* base = blob + (size_t)tile * tile_bytes(KS);
     float* f = reinterpret_cast<float*>(base);
-    f[r] = ok ? t.sx[s] : FAR;
-    f[TS + r] = ok ? t.sy[s] : 0.f;
-    f[2 * TS + r] = ok ? t.sr[s] : 0.f;
-    f[3 * TS + r] = ok ? t.sg[s] : 0.f;
-    f[4 * TS + r] = ok ? t.sb[s] : 0.f;
+    int pix = ok ? sample_pix[s] : 0;
+    if (pix < 0 || pix >= P) pix = 0;  // reported by the distance transform's seed pass
+    f[r] = ok ? (float)(pix % W) : FAR;
+    f[TS + r] = ok ? (float)(pix / W) : 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f[(2 + c) * TS + r] = ok ? img[(size_t)pix * 3 + c] : 0.f;
     for (int w = 0; w < KS; ++w) {
-        uint32_t bits = ok && 32 * w < k ? t.sbits[(size_t)w * n_samples + s] : 0u;
+        uint32_t bits = ok && w < Wk ? bitmask[(size_t)pix * Wk + w] : 0u;
         for (int c = k; c < k + 2; ++c)  // the columns of -|b_x|
             if (c >> 5 == w) bits |= 1u << (c & 31);
         uint8_t* slab = base + 5 * TS * 4 + w * TS * 32;
@@ -524,13 +524,14 @@ size_t plain_tile_bytes(int k, bool persample) {
     return (size_t)tile_bytes(persample ? steps_for(k) : 0);
 }
 
-cudaError_t launch_plain_tiles(const int32_t* d_label_off, int n_labels, int total_tiles, int k,
-                               int n_samples, bool persample, const SampleTables& t,
-                               cudaStream_t st) {
+cudaError_t launch_plain_tiles(const float* img, int H, int W, const uint32_t* bitmask, int k,
+                               int n_labels, const int32_t* d_label_off,
+                               const int32_t* sample_pix, int total_tiles, bool persample,
+                               uint8_t* blob, cudaStream_t st) {
     const long long n = (long long)total_tiles * TS;
     plain_tiles_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-        d_label_off, d_label_off + n_labels + 1, n_labels, total_tiles, t, n_samples, k,
-        persample ? steps_for(k) : 0, t.blob);
+        img, W, (long long)H * W, bitmask, (k + 31) / 32, d_label_off, d_label_off + n_labels + 1,
+        n_labels, sample_pix, total_tiles, k, persample ? steps_for(k) : 0, blob);
     return cudaGetLastError();
 }
 

@@ -455,28 +455,30 @@ __device__ void normalise_pixel(const TcArgs& a, const TcImage& im, int pix, con
     const long long P = (long long)im.H * im.W;
     float* nl = im.neglog + pix;
     if (!PERSAMPLE && im.rep) {  // factorised: the majority-co-support posterior
+        auto logit = [&](int i) {
+            const float rho = a.alpha * fmaxf(sqrtf((float)im.dist2[(size_t)i * P + pix]), a.d_min);
+            int h = 0;
+            for (int w = 0; w < a.Wk; ++w) h += __popc(bxp[w] ^ im.rep[i * a.Wk + w]);
+            return -LOG2E * (float)h / (a.kappa_beta * rho);
+        };
+        constexpr int NR = 8;  // labels whose logits stay in registers (the rest are formed again)
+        float t[NR];
         float tmax = -INFINITY;
-        for (int i = 0; i < im.n_labels; ++i) {
-            const float rho = a.alpha * fmaxf(sqrtf((float)im.dist2[(size_t)i * P + pix]), a.d_min);
-            int h = 0;
-            for (int w = 0; w < a.Wk; ++w) h += __popc(bxp[w] ^ im.rep[i * a.Wk + w]);
-            tmax = fmaxf(tmax, -LOG2E * (float)h / (a.kappa_beta * rho));
-        }
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+            if (i < im.n_labels) tmax = fmaxf(tmax, t[i] = logit(i));
+        for (int i = NR; i < im.n_labels; ++i) tmax = fmaxf(tmax, logit(i));
         float ts = 0.f;
-        for (int i = 0; i < im.n_labels; ++i) {
-            const float rho = a.alpha * fmaxf(sqrtf((float)im.dist2[(size_t)i * P + pix]), a.d_min);
-            int h = 0;
-            for (int w = 0; w < a.Wk; ++w) h += __popc(bxp[w] ^ im.rep[i * a.Wk + w]);
-            ts += ex2f(-LOG2E * (float)h / (a.kappa_beta * rho) - tmax);
-        }
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+            if (i < im.n_labels) ts += ex2f(t[i] - tmax);
+        for (int i = NR; i < im.n_labels; ++i) ts += ex2f(logit(i) - tmax);
         const float tl = tmax + log2f(ts);
-        for (int i = 0; i < im.n_labels; ++i) {
-            const float rho = a.alpha * fmaxf(sqrtf((float)im.dist2[(size_t)i * P + pix]), a.d_min);
-            int h = 0;
-            for (int w = 0; w < a.Wk; ++w) h += __popc(bxp[w] ^ im.rep[i * a.Wk + w]);
-            nl[(size_t)i * P] = nl[(size_t)i * P] -
-                                (-LOG2E * (float)h / (a.kappa_beta * rho) - tl) * LN2;
-        }
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+            if (i < im.n_labels) nl[(size_t)i * P] = nl[(size_t)i * P] - (t[i] - tl) * LN2;
+        for (int i = NR; i < im.n_labels; ++i)
+            nl[(size_t)i * P] = nl[(size_t)i * P] - (logit(i) - tl) * LN2;
     }
     float lmax = -INFINITY;
     for (int i = 0; i < im.n_labels; ++i) lmax = fmaxf(lmax, -nl[(size_t)i * P]);
@@ -1236,9 +1238,13 @@ __global__ void __launch_bounds__(128) refine_fp64_kernel(
     }
 }
 
-// Morton order of each label's samples in chunks of 4096 (one block per
-// chunk, bitonic sort of (key, index) pairs in shared memory): consecutive
-// 128-sample tiles then cover compact regions.
+// Morton order of each label's samples in chunks of 4096: consecutive 128-sample
+// tiles then cover compact regions. One block per chunk; bitonic sort of 64-bit
+// (key, index) values, four consecutive ones per thread: partners up to 2 apart
+// are in the thread, up to 64 apart in the warp (shuffles), and only the strides
+// from 128 on (15 of 78 steps) go through shared memory. Bound: issue and barrier
+// latency on one SM per chunk. Measured with chunks of 3100 samples: 23 us,
+// against 55 us with every step in shared memory.
 __device__ __forceinline__ uint32_t morton16(uint32_t v) {
     v &= 0xFFFFu;
     v = (v | (v << 8)) & 0x00FF00FFu;
@@ -1253,8 +1259,7 @@ __global__ void __launch_bounds__(1024) morton_sort_kernel(const int32_t* __rest
                                                            const int32_t* __restrict__ sample_pix,
                                                            int W, long long P,
                                                            int32_t* __restrict__ perm) {
-    __shared__ uint32_t key[4096];
-    __shared__ int32_t idx[4096];
+    __shared__ unsigned long long sv[4][1024];
     // chunk -> (label, first sample, count)
     int b = blockIdx.x, i = 0, start = 0, cnt = 0;
     for (; i < n_labels; ++i) {
@@ -1268,41 +1273,56 @@ __global__ void __launch_bounds__(1024) morton_sort_kernel(const int32_t* __rest
         b -= nch;
     }
     if (i == n_labels) return;
-    int n2 = 1;
+    int n2 = 4;
     while (n2 < cnt) n2 <<= 1;
-    for (int e = threadIdx.x; e < n2; e += blockDim.x) {
+    const int t = threadIdx.x;
+    unsigned long long v[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int e = 4 * t + r;
+        v[r] = ~0ull;
         if (e < cnt) {
-            const int sidx = start + e;
-            int pix = sample_pix[sidx];
+            int pix = sample_pix[start + e];
             if (pix < 0 || pix >= P) pix = 0;  // reported by the seed kernel
-            key[e] = morton16((uint32_t)(pix % W)) | (morton16((uint32_t)(pix / W)) << 1);
-            idx[e] = sidx;
-        } else {
-            key[e] = 0xFFFFFFFFu;
-            idx[e] = 0x7FFFFFFF;
+            const uint32_t key = morton16((uint32_t)(pix % W)) | (morton16((uint32_t)(pix / W)) << 1);
+            v[r] = (unsigned long long)key << 32 | (uint32_t)(start + e);
         }
     }
-    __syncthreads();
-    for (int kk = 2; kk <= n2; kk <<= 1)
-        for (int jj = kk >> 1; jj > 0; jj >>= 1) {
-            for (int e = threadIdx.x; e < n2; e += blockDim.x) {
-                const int partner = e ^ jj;
-                if (partner > e) {
-                    const bool up = (e & kk) == 0;
-                    const uint32_t ka = key[e], kb = key[partner];
-                    const int ia = idx[e], ib = idx[partner];
-                    const bool gt = ka > kb || (ka == kb && ia > ib);
-                    if (gt == up) {
-                        key[e] = kb;
-                        key[partner] = ka;
-                        idx[e] = ib;
-                        idx[partner] = ia;
-                    }
-                }
+    for (int kk = 2; kk <= n2; kk <<= 1) {
+        for (int jj = kk >> 1; jj >= 4; jj >>= 1) {
+            // (jj >= 4: the four values of a thread compare alike)
+            const bool keep_min = ((4 * t & kk) == 0) == ((4 * t & jj) == 0);
+            unsigned long long o[4];
+            if (jj >= 128) {
+                __syncthreads();
+#pragma unroll
+                for (int r = 0; r < 4; ++r) sv[r][t] = v[r];
+                __syncthreads();
+#pragma unroll
+                for (int r = 0; r < 4; ++r) o[r] = sv[r][t ^ (jj >> 2)];
+            } else {
+#pragma unroll
+                for (int r = 0; r < 4; ++r) o[r] = __shfl_xor_sync(0xffffffffu, v[r], jj >> 2);
             }
-            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < 4; ++r) v[r] = (o[r] < v[r]) == keep_min ? o[r] : v[r];
         }
-    for (int e = threadIdx.x; e < cnt; e += blockDim.x) perm[start + e] = idx[e];
+        auto order = [&](int x, int y) {
+            const bool up = ((4 * t + x) & kk) == 0;
+            const unsigned long long lo = min(v[x], v[y]), hi = max(v[x], v[y]);
+            v[x] = up ? lo : hi;
+            v[y] = up ? hi : lo;
+        };
+        if (kk >= 4) {
+            order(0, 2);
+            order(1, 3);
+        }
+        order(0, 1);
+        order(2, 3);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+        if (4 * t + r < cnt) perm[start + 4 * t + r] = (int32_t)(uint32_t)v[r];
 }
 
 // Sample tiles laid out as the bulk-copied part of a ring stage: the
@@ -1311,72 +1331,81 @@ __global__ void __launch_bounds__(1024) morton_sort_kernel(const int32_t* __rest
 // 8 + e), the texture slabs (b_j in {0, 1}) and the colour slab (hi/lo bf16
 // of I_j and of -C |I_j|^2); padded rows are zero. tile_xy receives each
 // tile slot's sample position x | y << 16, from which the producer forms
-// the location rows per pixel tile.
+// the location rows per pixel tile; the per-sample tables of the FP64
+// recompute are written on the way (every sample has one slot). One block per
+// tile. Bound: latency of the dependent loads (sample order, pixel, words).
+// Measured at 481 x 321, 10,000 samples: 5.6 us, against 15 us and a gather of
+// 5 us before it with one test per code.
 template <bool TEX8, int KS, bool PERSAMPLE>
-__global__ void build_tiles_kernel(const int32_t* __restrict__ label_off,
-                                   const int32_t* __restrict__ tile_off, int n_labels,
-                                   int total_tiles, SampleTables t, int n_samples, int k,
-                                   float Cc, const int32_t* __restrict__ perm,
-                                   uint8_t* __restrict__ blob, uint32_t* __restrict__ tile_xy,
-                                   float* __restrict__ imax2,
-                                   TcImage desc, TcImage* __restrict__ desc_dst) {
+__global__ void __launch_bounds__(BN) build_tiles_kernel(
+    const float* __restrict__ img, int W, long long P, const uint32_t* __restrict__ bitmask, int Wk,
+    const int32_t* __restrict__ sample_pix, const int32_t* __restrict__ label_off,
+    const int32_t* __restrict__ tile_off, int n_labels, int total_tiles, SampleTables t,
+    int n_samples, int k, float Cc, const int32_t* __restrict__ perm, uint8_t* __restrict__ blob,
+    uint32_t* __restrict__ tile_xy, float* __restrict__ imax2, TcImage desc,
+    TcImage* __restrict__ desc_dst) {
     using C = Cfg<TEX8, KS, PERSAMPLE>;
-    const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (gid == 0) *desc_dst = desc;  // this image's descriptor for the sum launch
-    if (gid >= (long long)total_tiles * BN) return;
-    const int tile = (int)(gid / BN), r = (int)(gid % BN);
+    constexpr int WMAX = 8;  // k <= 256
+    const int tile = blockIdx.x, r = threadIdx.x;
+    if (tile == 0 && r == 0) *desc_dst = desc;  // this image's descriptor for the sum launch
     int lo = 0, hi = n_labels - 1;  // label of this tile
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (tile_off[mid] <= tile) lo = mid; else hi = mid - 1;
     }
     const int i = lo;
-    const int first = label_off[i] + (tile - tile_off[i]) * BN;
-    const int pos = first + r;
+    const int pos = label_off[i] + (tile - tile_off[i]) * BN + r;
     const bool valid = pos < label_off[i + 1];
     const int s = valid ? perm[pos] : 0;
-    tile_xy[gid] = valid ? (uint32_t)t.sx[s] | ((uint32_t)t.sy[s] << 16) : 0u;
+    int pix = valid ? sample_pix[s] : 0;
+    if (pix < 0 || pix >= P) pix = 0;  // reported by seed_kernel; keep the tables finite
+    uint32_t bits[WMAX];
+#pragma unroll
+    for (int w = 0; w < WMAX; ++w)
+        bits[w] = valid && w < Wk ? bitmask[(size_t)pix * Wk + w] : 0u;
+    const float R = img[(size_t)pix * 3], G = img[(size_t)pix * 3 + 1], B = img[(size_t)pix * 3 + 2];
+    const int x = pix % W, y = pix / W;
+    if (valid) {
+        t.sx[s] = (float)x;
+        t.sy[s] = (float)y;
+        t.sr[s] = R;
+        t.sg[s] = G;
+        t.sb[s] = B;
+#pragma unroll
+        for (int w = 0; w < WMAX; ++w)
+            if (w < Wk) t.sbits[(size_t)w * n_samples + s] = bits[w];
+    }
+    tile_xy[(size_t)tile * BN + r] = valid ? (uint32_t)x | ((uint32_t)y << 16) : 0u;
+    // codes j0 .. j0 + 15 as bf16 1 / 0 pairs, and 4 codes as e4m3 bytes
+    auto bf16_pair = [](uint32_t b) { return (b & 1u) * 0x3F80u | (b >> 1 & 1u) * 0x3F800000u; };
+    auto e4m3_quad = [](uint32_t b) { return ((b & 15u) * 0x00204081u & 0x01010101u) * 0x38u; };
     // the bulk-copied part starts with L1's second half
     uint8_t* cp = blob + (size_t)tile * C::copy_bytes;
     uint32_t xw[4] = {0u, 0u, 0u, 0u};
-    if (PERSAMPLE && valid)
-        for (int e = 0, j = (TEX8 ? 32 : 16) * KS; j < k && e < EXT_MAX; ++e, ++j)
-            if ((t.sbits[(size_t)(j >> 5) * n_samples + s] >> (j & 31)) & 1u)
-                xw[e >> 1] |= 0x3F80u << (16 * (e & 1));
+    if (PERSAMPLE) {
+        constexpr int j0 = (TEX8 ? 32 : 16) * KS;
+        const uint32_t rest = (j0 >> 5) < WMAX ? bits[(j0 >> 5) < WMAX ? j0 >> 5 : 0] >> (j0 & 31) : 0u;
+        const uint32_t ext = rest & 0xFFu;  // EXT_MAX = 8 codes at most (bits beyond k are 0)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) xw[e] = bf16_pair(ext >> (2 * e));
+    }
     *reinterpret_cast<uint4*>(cp + tc::halves_off(r, 0)) = make_uint4(xw[0], xw[1], xw[2], xw[3]);
     uint8_t* st = cp + (C::tex_off - C::copy_off);
     if (PERSAMPLE) {
+#pragma unroll
         for (int sl = 0; sl < KS; ++sl) {
+            const uint32_t b = TEX8 ? bits[sl < WMAX ? sl : 0] : bits[(sl >> 1) < WMAX ? sl >> 1 : 0] >> (16 * (sl & 1));
             uint32_t wv[8];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                uint32_t word = 0;
-                if (TEX8) {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int j = 32 * sl + 4 * c + e;
-                        if (valid && j < k && ((t.sbits[(size_t)(j >> 5) * n_samples + s] >> (j & 31)) & 1u))
-                            word |= 0x38u << (8 * e);
-                    }
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int j = 16 * sl + 2 * c + e;
-                        if (valid && j < k && ((t.sbits[(size_t)(j >> 5) * n_samples + s] >> (j & 31)) & 1u))
-                            word |= 0x3F80u << (16 * e);
-                    }
-                }
-                wv[c] = word;
-            }
+            for (int c = 0; c < 8; ++c) wv[c] = TEX8 ? e4m3_quad(b >> (4 * c)) : bf16_pair(b >> (2 * c));
             *reinterpret_cast<uint4*>(st + sl * 4096 + tc::slab_off(r, 0)) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
             *reinterpret_cast<uint4*>(st + sl * 4096 + tc::slab_off(r, 16)) = make_uint4(wv[4], wv[5], wv[6], wv[7]);
         }
     }
     uint32_t pw[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    float i2 = 0.f;
     if (valid) {
-        const float R = t.sr[s], G = t.sg[s], B = t.sb[s];
-        const float i2 = fmaf(R, R, fmaf(G, G, B * B));
-        atomicMax(reinterpret_cast<int*>(imax2) + i, __float_as_int(i2));  // i2 >= 0
+        i2 = fmaf(R, R, fmaf(G, G, B * B));
         const float qv = -Cc * i2;
         uint16_t hr, lr, hg, lg, hb, lb, hq, lq;
         split_bf16(R, hr, lr);
@@ -1388,6 +1417,8 @@ __global__ void build_tiles_kernel(const int32_t* __restrict__ label_off,
         pw[4] = pack2(hb, lb); pw[5] = pack2(hb, lb);
         pw[6] = pack2(hq, lq); pw[7] = pack2(hq, lq);
     }
+    const int mx = __reduce_max_sync(0xffffffffu, __float_as_int(i2));  // i2 >= 0
+    if ((r & 31) == 0) atomicMax(reinterpret_cast<int*>(imax2) + i, mx);
     uint8_t* sc = cp + (C::col_off - C::copy_off);
     *reinterpret_cast<uint4*>(sc + tc::slab_off(r, 0)) = make_uint4(pw[0], pw[1], pw[2], pw[3]);
     *reinterpret_cast<uint4*>(sc + tc::slab_off(r, 16)) = make_uint4(pw[4], pw[5], pw[6], pw[7]);
@@ -1426,10 +1457,10 @@ cudaError_t tiles(const TcLaunch& L, cudaStream_t st) {
     d.first_ptile = L.first_ptile;
     cudaError_t e = cudaMemsetAsync(L.imax2, 0, sizeof(float) * L.n_labels, st);
     if (e != cudaSuccess) return e;
-    build_tiles_kernel<TEX8, KS, PERSAMPLE>
-        <<<(unsigned)(((long long)total_tiles * BN + 127) / 128), 128, 0, st>>>(
-            L.d_label_off, L.d_tile_off, L.n_labels, total_tiles, L.t, L.n_samples, L.k, Cc,
-            L.t.perm, L.blob, L.t.tile_xy, L.imax2, d, L.desc);
+    build_tiles_kernel<TEX8, KS, PERSAMPLE><<<(unsigned)total_tiles, BN, 0, st>>>(
+        L.img, L.W, (long long)L.H * L.W, L.bitmask, (L.k + 31) / 32, L.sample_pix, L.d_label_off,
+        L.d_tile_off, L.n_labels, total_tiles, L.t, L.n_samples, L.k, Cc, L.t.perm, L.blob,
+        L.t.tile_xy, L.imax2, d, L.desc);
     return cudaGetLastError();
 }
 
