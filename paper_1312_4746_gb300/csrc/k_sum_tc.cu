@@ -48,19 +48,20 @@
 //
 // Two persistent CTAs per SM (one where the shared-memory layout does not
 // fit twice).
-//   warps 8..11  producers: per stage, one bulk-copies (TMA) the
-//                pre-laid-out part of a sample tile (texture slabs, colour
-//                slab, the texture codes beyond the texture slabs), and all
-//                four write its location rows for this pixel tile (32
-//                samples each)
-//   warp 12      MMA issuer: D1 <- texture slabs + colour slab + location
+//   warp 8       producer: per stage, it bulk-copies (TMA) the pre-laid-out
+//                part of a sample tile (texture slabs, colour slab, the
+//                texture codes beyond the texture slabs), and writes its
+//                location rows for this pixel tile (two warps share the rows
+//                in the factorised form)
+//   last warp    MMA issuer: D1 <- texture slabs + colour slab + location
 //                slabs; TMEM double-buffered (2 x 128 columns per CTA), so
 //                one tile's MMAs run while the epilogue reads the previous
 //   warps 0..7   epilogue: writes the pixel-side colour and location rows
 //                of the NEXT item while it sums the current one (two label
 //                buffers), so that the MMAs run on across label boundaries;
 //                warp w reads lanes 32 (w % 4) .. +31 and columns
-//                64 (w / 4) .. +63 of each tile (16-column loads), merges the
+//                64 (w / 4) .. +63 of each tile (16-column loads, one ahead
+//                of the sums), merges the
 //                two column parts per item (16 warps of 32 columns in the
 //                one-CTA layout).
 // Every mbarrier wait is bounded by the global timer; on expiry the CTA sets
@@ -211,7 +212,15 @@ struct Cfg {
     static constexpr int EPQ = PAIR ? 2 : 4;                 // epilogue warps per TMEM lane quadrant
     static constexpr int EPI_WARPS = 4 * EPQ;
     static constexpr int CPW = BN / EPQ;                     // columns per epilogue warp per tile
-    static constexpr int NPROD = 4;                          // producer warps
+    // Producer warps. The sum is bound by instruction issue and a row of 32
+    // samples costs a producer about as much in waits and loop as in
+    // arithmetic: one warp per CTA forms all four rows of a tile (two in the
+    // factorised form, whose tiles take less time). Against four warps, with
+    // the registers this frees taken by the epilogue's loads in flight and the
+    // packed chunk sums: 481 x 321 412 -> 402 us, 1024 x 1024 36.5 -> 35.0 ms,
+    // 333 x 247 factorised 196 -> 189 us (one warp there: 191 us; two in the
+    // per-sample form: 404 us and 35.5 ms).
+    static constexpr int NPROD = PERSAMPLE ? 1 : 2;
     static constexpr int PRODUCER = EPI_WARPS;
     static constexpr int MMA_WARP = EPI_WARPS + NPROD;
     static constexpr int THREADS = (EPI_WARPS + NPROD + 1) * 32;
@@ -414,19 +423,20 @@ __device__ __forceinline__ uint64_t ex2x2(uint64_t v) {
 }
 __device__ __forceinline__ float lo32(uint64_t v) { return __uint_as_float((uint32_t)v); }
 __device__ __forceinline__ float hi32(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ float halves(uint64_t v) { return lo32(v) + hi32(v); }
 
 // Sum over 16 columns of one pixel row of 2^e, e = Bt D1 + k (log2 units,
 // shifted full exponents); r1 holds D1 as packed column pairs. Full chunk:
-// packed arithmetic; partial chunk: the first nv.
-__device__ __forceinline__ float sum16_full(const uint64_t (&r1)[8], uint64_t bt2, uint64_t k2) {
-    uint64_t acc0 = 0, acc1 = 0;  // (0.f, 0.f)
+// packed arithmetic, the sums of the even and of the odd columns; partial
+// chunk: the first nv.
+__device__ __forceinline__ uint64_t sum16_full(const uint64_t (&r1)[8], uint64_t bt2, uint64_t k2) {
+    uint64_t acc0 = ex2x2(fma2(bt2, r1[0], k2)), acc1 = ex2x2(fma2(bt2, r1[1], k2));
 #pragma unroll
-    for (int u = 0; u < 8; u += 2) {
+    for (int u = 2; u < 8; u += 2) {
         acc0 = add2(acc0, ex2x2(fma2(bt2, r1[u], k2)));
         acc1 = add2(acc1, ex2x2(fma2(bt2, r1[u + 1], k2)));
     }
-    const uint64_t t = add2(acc0, acc1);
-    return lo32(t) + hi32(t);
+    return add2(acc0, acc1);
 }
 __device__ __forceinline__ float sum16_part(const uint64_t (&r1)[8], int nv, uint64_t bt2,
                                             uint64_t k2) {
@@ -1021,27 +1031,37 @@ __global__ void __launch_bounds__((Cfg<TEX8, KS, PERSAMPLE, SOLO>::THREADS),
                 uint64_t x1[8];
                 bool released = false;
                 if (cbase + CPW <= nvalid) {  // warp-uniform: all columns valid
-                    float ts = 0.f;
+                    // chunk ch + 1 is in flight while chunk ch is summed
+                    uint64_t ts2 = 0;
+                    uint32_t xr[2][16];
+                    tc::tmem_ld16_issue(lb, xr[0]);
 #pragma unroll
                     for (int ch = 0; ch < CPW / 16; ++ch) {
-                        tc::tmem_ld16_wait_pk(lb + 16u * ch, x1);
-                        if (ch == CPW / 16 - 1) {
+                        tc::tmem_ld16_ready(xr[ch & 1]);
+                        if (ch + 1 < CPW / 16) {
+                            tc::tmem_ld16_issue(lb + 16u * (ch + 1), xr[(ch + 1) & 1]);
+                        } else {
                             // the last chunk is in registers: release the
                             // accumulator before its arithmetic
                             tc::fence_before_sync();
                             tc::mbar_arrive_elect(tmem_empty + b);
                             released = true;
                         }
-                        ts += sum16_full(x1, bt2, k2);
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            x1[u] = (uint64_t)xr[ch & 1][2 * u] |
+                                    ((uint64_t)xr[ch & 1][2 * u + 1] << 32);
+                        const uint64_t c2 = sum16_full(x1, bt2, k2);
+                        ts2 = ch ? add2(ts2, c2) : c2;
                     }
-                    two_sum(ts, S, Ccomp);
+                    two_sum(halves(ts2), S, Ccomp);
                 } else if (cbase < nvalid) {  // warp-uniform: the label's last tile
 #pragma unroll
                     for (int ch = 0; ch < CPW / 16; ++ch) {
                         const int nv = nvalid - cbase - 16 * ch;
                         if (nv > 0) {  // warp-uniform
                             tc::tmem_ld16_wait_pk(lb + 16u * ch, x1);
-                            const float ts = nv >= 16 ? sum16_full(x1, bt2, k2)
+                            const float ts = nv >= 16 ? halves(sum16_full(x1, bt2, k2))
                                                       : sum16_part(x1, nv, bt2, k2);
                             two_sum(ts, S, Ccomp);
                         }
