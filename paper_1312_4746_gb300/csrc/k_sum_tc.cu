@@ -48,12 +48,11 @@
 //
 // Two persistent CTAs per SM (one where the shared-memory layout does not
 // fit twice).
-//   warp 8       producer: per stage, it bulk-copies (TMA) the pre-laid-out
-//                part of a sample tile (texture slabs, colour slab, the
-//                texture codes beyond the texture slabs), and writes its
-//                location rows for this pixel tile (two warps share the rows
-//                in the factorised form)
-//   last warp    MMA issuer: D1 <- texture slabs + colour slab + location
+//   warps 8, 9   producers: per stage, one bulk-copies (TMA) the
+//                pre-laid-out part of a sample tile (texture slabs, colour
+//                slab, the texture codes beyond the texture slabs), and both
+//                write its location rows for this pixel tile (64 samples each)
+//   warp 10      MMA issuer: D1 <- texture slabs + colour slab + location
 //                slabs; TMEM double-buffered (2 x 128 columns per CTA), so
 //                one tile's MMAs run while the epilogue reads the previous
 //   warps 0..7   epilogue: writes the pixel-side colour and location rows
@@ -214,13 +213,14 @@ struct Cfg {
     static constexpr int CPW = BN / EPQ;                     // columns per epilogue warp per tile
     // Producer warps. The sum is bound by instruction issue and a row of 32
     // samples costs a producer about as much in waits and loop as in
-    // arithmetic: one warp per CTA forms all four rows of a tile (two in the
-    // factorised form, whose tiles take less time). Against four warps, with
-    // the registers this frees taken by the epilogue's loads in flight and the
-    // packed chunk sums: 481 x 321 412 -> 402 us, 1024 x 1024 36.5 -> 35.0 ms,
-    // 333 x 247 factorised 196 -> 189 us (one warp there: 191 us; two in the
-    // per-sample form: 404 us and 35.5 ms).
-    static constexpr int NPROD = PERSAMPLE ? 1 : 2;
+    // arithmetic: two warps per CTA form two rows each of a tile. Against four
+    // warps, with the registers this frees taken by the epilogue's loads in
+    // flight and the packed chunk sums: 481 x 321 412 -> 404 us, 1024 x 1024
+    // 36.5 -> 35.5 ms, 333 x 247 factorised 196 -> 189 us. One warp is faster
+    // still by up to 2% where location rows are truncations (402 us, 35.0 ms), but
+    // where they aren't (sides above LOC_NARROW) it holds the MMAs up: 3000 x 400,
+    // BF16, 3.59 ms against 3.21 with two and 3.39 with four.
+    static constexpr int NPROD = 2;
     static constexpr int PRODUCER = EPI_WARPS;
     static constexpr int MMA_WARP = EPI_WARPS + NPROD;
     static constexpr int THREADS = (EPI_WARPS + NPROD + 1) * 32;
