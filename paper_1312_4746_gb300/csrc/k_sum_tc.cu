@@ -211,7 +211,7 @@ struct Cfg {
     static constexpr int EPQ = PAIR ? 2 : 4;                 // epilogue warps per TMEM lane quadrant
     static constexpr int EPI_WARPS = 4 * EPQ;
     static constexpr int CPW = BN / EPQ;                     // columns per epilogue warp per tile
-    // Producer warps. The sum is bound by instruction issue and a row of 32
+    // Producer warps. The sum's time follows its instructions, and a row of 32
     // samples costs a producer about as much in waits and loop as in
     // arithmetic: two warps per CTA form two rows each of a tile. Against four
     // warps, with the registers this frees taken by the epilogue's loads in
@@ -365,7 +365,7 @@ __device__ __forceinline__ void loc_row_b(uint32_t w, int cx, int cy, bool valid
 // one by one (eight conversions a row, in the unit that the exponentials need).
 // fx, fy: -(2^24 + 2 cx), -(2^24 + 2 cy). At 481 x 321 the producers' rows were
 // 514 of about 2700 warp instructions per sample tile, now about 390; the whole
-// data term went from 433 to 429 us there, from 37.8 to 36.7 ms at 1024 x 1024.
+// data term went from 444 to 429 us there, from 37.8 to 36.7 ms at 1024 x 1024.
 constexpr int LOC_NARROW = 2880;  // 2 (2880 + 8)^2 < 2^24
 __device__ __forceinline__ void loc_row_narrow(uint32_t w, float fx, float fy, uint4& l0a, uint4& l0b,
                                                uint4& l1a) {
