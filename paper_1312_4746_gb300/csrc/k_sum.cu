@@ -36,6 +36,7 @@
 #include <type_traits>
 
 #include "internal.h"
+#include "mma_phase.h"
 #include "tc_ptx.cuh"
 
 namespace {
@@ -173,11 +174,11 @@ __global__ void __launch_bounds__(256) plain_tiles_kernel(
     }
 }
 
-// Waits for the phase with the given parity, for PLAIN_WAIT_NS at most.
-__device__ __forceinline__ bool plain_wait(uint64_t* bar, uint32_t parity) {
+// Waits for the MMAs of one tile, for PLAIN_WAIT_NS at most.
+__device__ __forceinline__ bool plain_wait(uint64_t* bars, MmaPhase p) {
     uint64_t deadline = 0;
     for (uint32_t n = 0;; ++n) {
-        if (tc::mbar_try_wait(bar, parity, 1000u)) return true;
+        if (tc::mbar_try_wait(bars + p.bar, p.parity, 1000u)) return true;
         if ((n & 63u) == 63u) {
             const uint64_t now = tc::globaltimer();
             if (deadline == 0) deadline = now + PLAIN_WAIT_NS;
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
         tc::fence_after_sync();
         tmem = *s_tmem;
     }
-    uint32_t it0 = 0;  // tiles before this unit
+    uint32_t it0 = 0;  // tiles issued before this unit
     bool ok = true;
 
     for (long long unit = blockIdx.x; ok && unit < n_units; unit += gridDim.x) {
@@ -301,9 +302,10 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
 
         // the exponents and sums of tile T
         auto sum_tile = [&](int T) {
-            const uint32_t it = it0 + (uint32_t)T, b = it & 1u;
+            const uint32_t it = it0 + (uint32_t)T, b = mma_phase(it).bar;
             if (TEX) {
-                ok = plain_wait(bars + b, (it >> 1) & 1u);
+                // (one decision per warp: the load below takes the whole warp)
+                ok = __all_sync(0xffffffffu, plain_wait(bars, mma_phase(it)));
                 if (!ok) return;
                 tc::fence_after_sync();
             }
@@ -381,7 +383,8 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
             }
         };
 
-        for (int T = 0; T <= nt; ++T) {
+        int T = 0;
+        for (; T <= nt; ++T) {
             if (T < nt) asm volatile("cp.async.wait_group 1;" ::: "memory");
             if (TEX) {
                 tc::fence_proxy_async_smem();  // this thread's copies and operand rows
@@ -392,7 +395,7 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
             if (T < nt) {
                 if (TEX && tid == 0) {
                     tc::fence_after_sync();
-                    const uint32_t b = (it0 + (uint32_t)T) & 1u;
+                    const uint32_t b = mma_phase(it0 + (uint32_t)T).bar;
                     const uint32_t al = tc::desc_lo(smem);
                     const uint32_t bl = tc::desc_lo(ring + (T % STAGES) * TB + 5 * TS * 4);
                     constexpr uint32_t id = tc::idesc(128, TS, 0, 0);
@@ -409,7 +412,7 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
             }
             if (T > 0) sum_tile(T - 1);
         }
-        it0 += (uint32_t)nt;
+        it0 += (uint32_t)min(T, nt);  // (a wait that gave up leaves the loop before tile T)
 
         // the pixel's two threads: common maximum, scaled sums
         if (hf == 1)
@@ -448,9 +451,10 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
     if (TEX) {
         if (!ok && tid == 0) {
             if (atomicCAS(a.d_err, 0, CS_DEVERR_TIMEOUT) == 0) a.d_err[1] = 51;
-            // MMAs still in flight: they must finish before the tensor memory is freed
-            plain_wait(bars, 0);
-            plain_wait(bars + 1, 0);
+            // MMAs still in flight: they must finish before the tensor memory is
+            // freed and the operands' shared memory goes to another CTA
+            MmaPhase last;
+            if (mma_last(it0, last)) plain_wait(bars, last);
         }
         tc::fence_before_sync();
         __syncthreads();
