@@ -113,6 +113,14 @@ cs_status cs_set_error(cs_ctx* ctx, cs_status code, const char* fmt, ...);
 cs_status cs_ensure_scratch(cs_ctx* ctx, size_t bytes);
 cs_status cs_check_launch(cs_ctx* ctx, const char* what);
 
+// Dynamic shared memory limit of a kernel, before its launches. The limit belongs to
+// the kernel on the device, not to a launch or a context: `most` is the largest that
+// any call needs, so that a call cannot lower the limit between another thread's
+// setting it and its launches.
+inline cudaError_t cs_smem_limit(const void* kernel, size_t most) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // ---- launchers (each enqueues kernels on `st`; returns cudaError_t) -------
 
 // Patches, codes, co-support bitmasks (FP32 with a rigorous guard band and

@@ -1111,8 +1111,7 @@ template <int P>
 cudaError_t launch_tc_p(const CodesArgs& a, cudaStream_t st) {
     const int np = ct_np(a.k);
     const size_t smem = ct_smem<P>(np);
-    cudaError_t e = cudaFuncSetAttribute(codes_tc_kernel<P>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cs_smem_limit((const void*)codes_tc_kernel<P>, ct_smem<P>(256));
     if (e != cudaSuccess) return e;
     const int total = 3 * ct_ks(P) * np * 16;
     omega_split_kernel<<<(total + 255) / 256, 256, 0, st>>>(a.omega, a.k, P * P, ct_ks(P), np,
@@ -1137,8 +1136,7 @@ cudaError_t launch_tc_p(const CodesArgs& a, cudaStream_t st) {
     }
     const size_t floor_b = 233472 / (per_sm + 1) - 1024 + 16;  // no further CTA fits
     if (psmem < floor_b) psmem = floor_b;
-    e = cudaFuncSetAttribute(codes_tcp_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)psmem);
+    e = cs_smem_limit((const void*)codes_tcp_kernel<P>, 233472 - 1024);  // one CTA per SM takes all
     if (e != cudaSuccess) return e;
     int dev = 0, n_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;

@@ -926,10 +926,6 @@ __global__ void calib_kernel(const float* __restrict__ Z, const float* __restric
     atomicMax(reinterpret_cast<int*>(eta), __float_as_int(mx));
 }
 
-cudaError_t set_smem(const void* fn, size_t bytes) {
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 }  // namespace
 
 int mlp_param_count(int nin, int n) { return off_of(nin, n).np; }
@@ -959,7 +955,7 @@ cudaError_t launch_mlp_train(const unsigned char* image, int nin, int n, const f
                              int* d_err, uint64_t wait_ns, cudaStream_t st) {
     const Dims dm = dims_of(nin, n);
     const size_t smem = train_layout(dm.K0, dm.NOp).total;
-    cudaError_t e = set_smem((const void*)mlp_train_kernel, smem);
+    cudaError_t e = cs_smem_limit((const void*)mlp_train_kernel, train_layout(64, CS_MAX_LABELS).total);
     if (e != cudaSuccess) return e;
     TrainArgs a{image, nin, n, X, T, n_rows, start, batch, part, mlp_part_stride(nin, n), d_err,
                 wait_ns ? wait_ns : MLP_WAIT_NS};
@@ -989,7 +985,8 @@ cudaError_t launch_mlp_forward(const unsigned char* image, int nin, int n, const
                                float* Z, int n_sm, int* d_err, uint64_t wait_ns, cudaStream_t st) {
     const Dims dm = dims_of(nin, n);
     const size_t smem = fwd_layout(dm.K0, dm.NOp).total;
-    cudaError_t e = set_smem((const void*)mlp_fwd_kernel<SRC_ROWS>, smem);
+    cudaError_t e =
+        cs_smem_limit((const void*)mlp_fwd_kernel<SRC_ROWS>, fwd_layout(64, CS_MAX_LABELS).total);
     if (e != cudaSuccess) return e;
     FwdArgs a{};
     a.image = image;
@@ -1007,7 +1004,8 @@ cudaError_t launch_mlp_forward(const unsigned char* image, int nin, int n, const
 cudaError_t launch_surrogate_eval(const SurrogateEvalArgs& s, cudaStream_t st) {
     const Dims dm = dims_of(s.nin, s.n);
     const size_t smem = fwd_layout(dm.K0, dm.NOp).total;
-    cudaError_t e = set_smem((const void*)mlp_fwd_kernel<SRC_EVAL>, smem);
+    cudaError_t e =
+        cs_smem_limit((const void*)mlp_fwd_kernel<SRC_EVAL>, fwd_layout(64, CS_MAX_LABELS).total);
     if (e != cudaSuccess) return e;
     FwdArgs a{};
     a.image = s.image;

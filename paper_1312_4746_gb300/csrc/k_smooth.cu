@@ -412,14 +412,18 @@ __global__ void __launch_bounds__(TX* TY) smooth_texture_kernel(
 }
 
 template <int P, int NB>
+constexpr size_t texture_smem(int k, int n_labels) {
+    constexpr int N = P * P, NP = (N + 3) & ~3, TW = TX + P - 1, TH = TPX * TY + P - 1;
+    return sizeof(float) * ((size_t)32 * NP + (size_t)k * NB + 2 * TW * TH + NP +
+                            (size_t)n_labels * TPX * TX * TY);
+}
+
+template <int P, int NB>
 cudaError_t texture_p(const SmoothArgs& a, cudaStream_t st) {
-    constexpr int N = P * P, NP = (N + 3) & ~3, TW = TX + P - 1;
-    constexpr int TH = TPX * TY + P - 1;
-    const size_t smem =
-        sizeof(float) * ((size_t)32 * NP + (size_t)a.k * NB + 2 * TW * TH + ((N + 3) & ~3) +
-                         (size_t)a.n_labels * TPX * TX * TY);
-    cudaError_t e = cudaFuncSetAttribute(smooth_texture_kernel<P, NB>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = texture_smem<P, NB>(a.k, a.n_labels);
+    // (likelihoods take at most 256 codes)
+    cudaError_t e = cs_smem_limit((const void*)smooth_texture_kernel<P, NB>,
+                                  texture_smem<P, NB>(256, CS_MAX_LABELS));
     if (e != cudaSuccess) return e;
     dim3 grd((a.W + TX - 1) / TX, (a.H + TPX * TY - 1) / (TPX * TY));
     smooth_texture_kernel<P, NB><<<grd, TX * TY, smem, st>>>(

@@ -550,11 +550,9 @@ int grid_for(long long N, int n_sm) {
     return (int)(need < 1 ? 1 : need < cap ? need : cap);
 }
 
-cudaError_t set_smem(const void* f, size_t bytes) {
-    return bytes > 48 * 1024
-               ? cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)
-               : cudaSuccess;
-}
+// dynamic shared memory of the median kernel and of the kernels that hold k x cpad(NC) centres
+constexpr size_t median_smem(int n) { return sizeof(unsigned) * ((size_t)n * HB + LCAP) + LCAP; }
+constexpr size_t centres_smem(int k, int nc) { return sizeof(float) * (size_t)k * cpad(nc); }
 
 }  // namespace
 
@@ -579,8 +577,8 @@ cudaError_t launch_kmeans(const KmeansArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_kmedians(const KmediansArgs& a, cudaStream_t st) {
-    const size_t hbytes = sizeof(unsigned) * ((size_t)a.n * HB + LCAP) + LCAP;
-    cudaError_t e = set_smem((const void*)class_median_kernel, hbytes);
+    const size_t hbytes = median_smem(a.n);
+    cudaError_t e = cs_smem_limit((const void*)class_median_kernel, median_smem(CS_MAX_CLASSES));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute((const void*)class_median_kernel,
                                  cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -590,8 +588,9 @@ cudaError_t launch_kmedians(const KmediansArgs& a, cudaStream_t st) {
                                                                    a.C);
     return with_classes(a.n, [&](auto nc) {
         constexpr int NC = decltype(nc)::value;
-        const size_t smem = sizeof(float) * (size_t)a.k * cpad(NC);
-        cudaError_t e2 = set_smem((const void*)kmedians_assign_kernel<NC>, smem);
+        const size_t smem = centres_smem(a.k, NC);
+        cudaError_t e2 =
+            cs_smem_limit((const void*)kmedians_assign_kernel<NC>, centres_smem(CS_MAX_K, NC));
         if (e2 != cudaSuccess) return e2;
         const int g = grid_for(a.N, a.n_sm);
         for (int it = 0; it < a.iterations; ++it) {
@@ -610,8 +609,8 @@ cudaError_t launch_kmedians(const KmediansArgs& a, cudaStream_t st) {
 cudaError_t launch_unsup_final(const UnsupFinalArgs& a, cudaStream_t st) {
     return with_classes(a.nt, [&](auto nc) {
         constexpr int NC = decltype(nc)::value;
-        const size_t smem = sizeof(float) * (size_t)a.k * cpad(NC);
-        cudaError_t e = set_smem((const void*)unsup_final_kernel<NC>, smem);
+        const size_t smem = centres_smem(a.k, NC);
+        cudaError_t e = cs_smem_limit((const void*)unsup_final_kernel<NC>, centres_smem(CS_MAX_K, NC));
         if (e != cudaSuccess) return e;
         unsup_final_kernel<NC><<<grid_for(a.P, a.n_sm), UB, smem, st>>>(
             a.img, a.P, a.V, a.k, a.Ccol, a.nc, a.Ctex, a.nt, a.inv2s2, a.inv_beta, a.neglog,
