@@ -169,6 +169,9 @@ cs_status cs_sync_status(cs_ctx* ctx, void* stream);
  *                               MMA-issuing thread of the last CTA waits,
  *                               before it issues anything, on a barrier that
  *                               nothing completes
+ *             CS_STALL_PLAIN    the plain FP32 sum (cs_likelihood or
+ *                               cs_data_term with CS_FP32 and
+ *                               CS_MODE_PERSAMPLE): as CS_STALL_SUM
  * The other waits of that launch then run out after limit_ns (or see the
  * abort flag the first one raised); the launch ends, cs_sync_status returns
  * CS_ERR_TIMEOUT, the stalled launch's outputs are undefined, and the
@@ -178,6 +181,7 @@ cs_status cs_sync_status(cs_ctx* ctx, void* stream);
 #define CS_STALL_NONE 0
 #define CS_STALL_SEGMENT 1
 #define CS_STALL_SUM 2
+#define CS_STALL_PLAIN 4
 cs_status cs_test_wait(cs_ctx* ctx, int64_t limit_ns, int stall);
 
 /*

@@ -36,6 +36,7 @@ CODES_TC = 2
 STALL_NONE = 0
 STALL_SEGMENT = 1
 STALL_SUM = 2
+STALL_PLAIN = 4
 
 # every symbol include/cosparse.h declares
 EXPORTS = (

@@ -412,7 +412,7 @@ cs_status cs_refined_count(cs_ctx* ctx, int32_t* count, void* stream) {
 cs_status cs_test_wait(cs_ctx* ctx, int64_t limit_ns, int stall) {
     if (!ctx) return cs_set_error(nullptr, CS_ERR_INVALID_ARG, "cs_test_wait: ctx is NULL");
     if (limit_ns < 0 || (stall != CS_STALL_NONE && stall != CS_STALL_SEGMENT &&
-                         stall != CS_STALL_SUM))
+                         stall != CS_STALL_SUM && stall != CS_STALL_PLAIN))
         return cs_set_error(ctx, CS_ERR_INVALID_ARG, "cs_test_wait: limit %lld ns, stall %d",
                             (long long)limit_ns, stall);
     ctx->wait_ns = (unsigned long long)limit_ns;
@@ -648,6 +648,7 @@ SumArgs cs_sum_args(cs_ctx* ctx, const LikPlan& L, const float* img, const uint3
     a.neglog = neglog;
     a.post = post;
     a.d_err = ctx->d_err;
+    a.wait_ns = ctx->wait_ns;
     return a;
 }
 
@@ -727,8 +728,11 @@ static cudaError_t enqueue_sum(cs_ctx* ctx, const LikPlan& L, const float* img,
     if (e == cudaSuccess && dist_ready) e = cudaStreamWaitEvent(st, dist_ready, 0);
     if (e != cudaSuccess) return e;
     StageTimer tm(ctx, CS_STAGE_SUM, st);
-    if (!L.tc_form) return launch_sum_plain(cs_sum_args(ctx, L, img, bitmask, prm, neglog, post), st);
-    return launch_sum_tc_run(T, st);
+    if (L.tc_form) return launch_sum_tc_run(T, st);
+    SumArgs a = cs_sum_args(ctx, L, img, bitmask, prm, neglog, post);
+    a.stall = L.persample && ctx->stall == CS_STALL_PLAIN;
+    if (a.stall) ctx->stall = CS_STALL_NONE;
+    return launch_sum_plain(a, st);
 }
 
 extern "C" {

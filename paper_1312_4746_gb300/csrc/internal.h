@@ -49,7 +49,7 @@ struct cs_ctx {
     bool profiling = false;
     // timeout-path test hook (cs_test_wait): wait limit of the bounded device
     // waits (0: the kernels' own 1 s) and a one-shot stall of the next
-    // solver or tensor-core sum launch
+    // launch of one kernel
     unsigned long long wait_ns = 0;
     int stall = 0;
     std::vector<StageRecord> records;
@@ -310,6 +310,8 @@ struct SumArgs {
     int list_cap = 0;
     float* T_out = nullptr;
     int* d_err = nullptr;  // device error word (a wait for the tensor cores that gave up)
+    unsigned long long wait_ns = 0;  // limit of each wait for the tensor cores (0: 1 s)
+    bool stall = false;  // timeout-path test: the last block waits for what nothing completes
 };
 // (over the sample tiles of launch_plain_tiles, whose offsets per label follow
 // the label offsets at d_label_off + n_labels + 1)

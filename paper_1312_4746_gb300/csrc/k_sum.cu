@@ -48,7 +48,7 @@ constexpr float LOG2E = 1.4426950408889634f;
 constexpr float LN2 = 0.6931471805599453f;
 constexpr float FAR = 1.0e18f;
 constexpr float LOWEST = -3.0e38f;
-constexpr uint64_t PLAIN_WAIT_NS = 1000000000ull;  // limit of a wait for an MMA
+constexpr uint64_t PLAIN_WAIT_NS = 1000000000ull;  // default limit of a wait for an MMA
 
 // 32-column steps of the texture operands: k codes and the two columns of -|b_x|
 __host__ __device__ constexpr int steps_for(int k) { return (k + 2 + 31) / 32; }
@@ -174,14 +174,14 @@ __global__ void __launch_bounds__(256) plain_tiles_kernel(
     }
 }
 
-// Waits for the MMAs of one tile, for PLAIN_WAIT_NS at most.
-__device__ __forceinline__ bool plain_wait(uint64_t* bars, MmaPhase p) {
+// Waits for the MMAs of one tile, for wait_ns (0: PLAIN_WAIT_NS) at most.
+__device__ __forceinline__ bool plain_wait(uint64_t* bars, MmaPhase p, uint64_t wait_ns) {
     uint64_t deadline = 0;
     for (uint32_t n = 0;; ++n) {
         if (tc::mbar_try_wait(bars + p.bar, p.parity, 1000u)) return true;
         if ((n & 63u) == 63u) {
             const uint64_t now = tc::globaltimer();
-            if (deadline == 0) deadline = now + PLAIN_WAIT_NS;
+            if (deadline == 0) deadline = now + (wait_ns ? wait_ns : PLAIN_WAIT_NS);
             else if (now > deadline) return false;
         }
     }
@@ -201,8 +201,9 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* ring = smem + off_ring(KS, PT);
     float* xchg = reinterpret_cast<float*>(smem + off_xchg(KS, PT));  // [3][PT][128]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + off_bars(KS, PT));  // [2] MMA commits
-    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 2);
+    // [2] MMA commits, then one that nothing completes (the timeout-path test)
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + off_bars(KS, PT));
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 3);
     const long long P = (long long)a.H * a.W;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int row = 32 * (warp & 3) + lane, hf = warp >> 2;  // operand row, column half
@@ -221,6 +222,7 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
         if (tid == 0) {
             tc::mbar_init(bars, 1);
             tc::mbar_init(bars + 1, 1);
+            tc::mbar_init(bars + 2, 1);
             tc::fence_mbar_init();
         }
         if (warp == 0) {
@@ -234,6 +236,9 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
     }
     uint32_t it0 = 0;  // tiles issued before this unit
     bool ok = true;
+    // the timeout-path test: the last block gives up before it issues anything
+    if (TEX && a.stall && blockIdx.x == gridDim.x - 1)
+        ok = __syncthreads_and(tid != 0 || plain_wait(bars, MmaPhase{2u, 0u}, a.wait_ns));
 
     for (long long unit = blockIdx.x; ok && unit < n_units; unit += gridDim.x) {
         const int i = (int)(unit % a.n_labels);
@@ -305,7 +310,7 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
             const uint32_t it = it0 + (uint32_t)T, b = mma_phase(it).bar;
             if (TEX) {
                 // (one decision per warp: the load below takes the whole warp)
-                ok = __all_sync(0xffffffffu, plain_wait(bars, mma_phase(it)));
+                ok = __all_sync(0xffffffffu, plain_wait(bars, mma_phase(it), a.wait_ns));
                 if (!ok) return;
                 tc::fence_after_sync();
             }
@@ -454,7 +459,7 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
             // MMAs still in flight: they must finish before the tensor memory is
             // freed and the operands' shared memory goes to another CTA
             MmaPhase last;
-            if (mma_last(it0, last)) plain_wait(bars, last);
+            if (mma_last(it0, last)) plain_wait(bars, last, a.wait_ns);
         }
         tc::fence_before_sync();
         __syncthreads();

@@ -1,0 +1,68 @@
+"""The give-up path of the bounded waits in the forms that test_gpu_timeout.py's
+calls do not reach: the plain FP32 sum's wait for its tensor-core products. As there: the one-shot hook makes
+one wait run out before anything is in flight, the call reports the timeout within
+the shortened limit, and the next call gives the earlier bits.
+"""
+import re
+import time
+
+import numpy as np
+import pytest
+
+from paper_1312_4746_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+LIMIT_NS = 20_000_000  # 20 ms: far above any normal wait of these launches
+
+
+@pytest.fixture(scope="module")
+def env(cuda_lib):
+    import torch
+
+    import paper_1312_4746_gb300 as cs
+
+    ctx = cs.Context(0)
+    yield cs, ctx, torch
+    ctx.test_wait(0, cs.STALL_NONE)
+    ctx.close()
+
+
+def _stalled(cs, ctx, stall, call):
+    """Runs `call` with the stall armed: the site of the wait that gave up."""
+    ctx.test_wait(LIMIT_NS, stall)
+    t0 = time.perf_counter()
+    call()
+    with pytest.raises(cs.CsError) as ei:
+        ctx.sync()
+    dt = time.perf_counter() - t0
+    ctx.test_wait(0, cs.STALL_NONE)
+    assert ei.value.status == cs.CS_ERR_TIMEOUT, ei.value
+    assert dt < 0.5, dt  # the shortened limit, not the default 1 s
+    return int(re.search(r"site (\d+)", str(ei.value)).group(1))
+
+
+@pytest.mark.parametrize("H,W", [(64, 96), (152, 257)])  # one and two operand tiles per block
+def test_plain_sum(env, H, W):
+    cs, ctx, torch = env
+    pr = synth.make_problem(H, W, 4, [70, 5, 64, 130], p=5, k=50, seed=77)
+    img, om, mask, smp = (torch.from_numpy(np.ascontiguousarray(a)).to("cuda:0")
+                          for a in (pr.image, pr.omega, pr.mask, pr.sample_pix))
+    prm = cs.Params.from_synth(pr.params)
+    bits = ctx.codes(img, om, mask, prm)["bitmask"]
+
+    def call(p=prm):
+        return ctx.likelihood(img, bits, 50, pr.label_off, smp, p)["neglog"]
+
+    ref = call()
+    ctx.sync()
+    assert _stalled(cs, ctx, cs.STALL_PLAIN, call) == 51
+    assert torch.equal(call(), ref)
+    # forms without that wait leave the stall armed
+    ctx.test_wait(LIMIT_NS, cs.STALL_PLAIN)
+    call(cs.Params.from_synth(pr.params, mode=cs.MODE_FACTORISED))
+    call(cs.Params.from_synth(pr.params, precision=cs.FP8))
+    ctx.sync()
+    ctx.test_wait(0, cs.STALL_NONE)
+    assert torch.equal(call(), ref)
+    ctx.sync()
