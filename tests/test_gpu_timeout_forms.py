@@ -1,5 +1,7 @@
 """The give-up path of the bounded waits in the forms that test_gpu_timeout.py's
-calls do not reach: the plain FP32 sum's wait for its tensor-core products. As there: the one-shot hook makes
+calls do not reach: the solver's tile form with a label cost (which also waits for
+the blocks' sums) and its general form (grid barriers; more than 16 labels), and the
+plain FP32 sum's wait for its tensor-core products. As there: the one-shot hook makes
 one wait run out before anything is in flight, the call reports the timeout within
 the shortened limit, and the next call gives the earlier bits.
 """
@@ -40,6 +42,21 @@ def _stalled(cs, ctx, stall, call):
     assert ei.value.status == cs.CS_ERR_TIMEOUT, ei.value
     assert dt < 0.5, dt  # the shortened limit, not the default 1 s
     return int(re.search(r"site (\d+)", str(ei.value)).group(1))
+
+
+@pytest.mark.parametrize("n,nu", [(3, 0.0), (3, 30.0), (16, 30.0), (17, 0.0), (17, 30.0)])
+def test_segment_forms(env, n, nu):
+    cs, ctx, torch = env
+    g = torch.Generator(device="cuda:0").manual_seed(n)
+    f = 3.0 * torch.rand((n, 64, 96), generator=g, device="cuda:0")
+    img = torch.rand((64, 96, 3), generator=g, device="cuda:0")
+    sp = cs.SegParams.default(lam=2.0, nu=nu, iterations=20)
+    ref = ctx.segment(f, img, sp)
+    ctx.sync()
+    assert _stalled(cs, ctx, cs.STALL_SEGMENT, lambda: ctx.segment(f, img, sp)) == 41
+    out = ctx.segment(f, img, sp)
+    ctx.sync()
+    assert torch.equal(out["u"], ref["u"]) and torch.equal(out["labels"], ref["labels"])
 
 
 @pytest.mark.parametrize("H,W", [(64, 96), (152, 257)])  # one and two operand tiles per block
