@@ -846,6 +846,13 @@ __device__ __forceinline__ bool cp_wait(uint64_t* bar, uint32_t parity, volatile
     return false;
 }
 
+// The same by a whole warp, with one outcome: lanes on either side of the deadline
+// would part before the barriers and warp-wide loads that follow.
+__device__ __forceinline__ bool cp_wait_warp(uint64_t* bar, uint32_t parity,
+                                             volatile int* abort_flag, int* d_err, int site) {
+    return __all_sync(0xffffffffu, cp_wait(bar, parity, abort_flag, d_err, site));
+}
+
 template <int P>
 __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kernel(
     const float* __restrict__ img, int H, int W, const uint8_t* __restrict__ blob, int k, int np,
@@ -963,7 +970,7 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
                                      5 * KS * 4.76837158203125e-07f * 0.0079f;
             const float ebase = (ds + EPS_TC * (1.f + ds)) * 1.25f;
             // the A operand is free once the previous tile's MMAs have read it
-            if (!cp_wait(a_empty, (uint32_t)((kk & 1) ^ 1), abort_flag, d_err, 23)) break;
+            if (!cp_wait_warp(a_empty, (uint32_t)((kk & 1) ^ 1), abort_flag, d_err, 23)) break;
 #pragma unroll
             for (int sl = 0; sl < KS; ++sl) {
                 uint32_t w1[8], w2[8], w3[8];
@@ -1006,7 +1013,7 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
             if (lane == 0) tc::mbar_arrive(a_full);
             // this pixel's parameters for the epilogue
             const int pb = kk & 1;
-            if (!cp_wait(p_empty + pb, (uint32_t)(((kk >> 1) & 1) ^ 1), abort_flag, d_err, 24)) break;
+            if (!cp_wait_warp(p_empty + pb, (uint32_t)(((kk >> 1) & 1) ^ 1), abort_flag, d_err, 24)) break;
             prm[pb * 128 + r] = make_int4(live ? pix : -1, whole ? 1 : 0, __float_as_int(ebase), 0);
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(p_full + pb);
@@ -1019,11 +1026,11 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
         int kk = 0;
         for (int T = blockIdx.x; T < ntiles; T += gridDim.x, ++kk) {
             const int b = kk & 1;
-            if (!cp_wait(p_full + b, (uint32_t)((kk >> 1) & 1), abort_flag, d_err, 25)) break;
+            if (!cp_wait_warp(p_full + b, (uint32_t)((kk >> 1) & 1), abort_flag, d_err, 25)) break;
             const int4 pp = prm[b * 128 + 32 * q + lane];
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(p_empty + b);
-            if (!cp_wait(t_full + b, (uint32_t)((kk >> 1) & 1), abort_flag, d_err, 26)) break;
+            if (!cp_wait_warp(t_full + b, (uint32_t)((kk >> 1) & 1), abort_flag, d_err, 26)) break;
             tc::fence_after_sync();
             const bool live = pp.x >= 0, whole = pp.y != 0;
             const int pix = live ? pp.x : 0;
