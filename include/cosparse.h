@@ -172,6 +172,8 @@ cs_status cs_sync_status(cs_ctx* ctx, void* stream);
  *             CS_STALL_PLAIN    the plain FP32 sum (cs_likelihood or
  *                               cs_data_term with CS_FP32 and
  *                               CS_MODE_PERSAMPLE): as CS_STALL_SUM
+ *             CS_STALL_CODES    the tensor-core codes (cs_codes or cs_data_term):
+ *                               as CS_STALL_SUM
  * The other waits of that launch then run out after limit_ns (or see the
  * abort flag the first one raised); the launch ends, cs_sync_status returns
  * CS_ERR_TIMEOUT, the stalled launch's outputs are undefined, and the
@@ -182,6 +184,7 @@ cs_status cs_sync_status(cs_ctx* ctx, void* stream);
 #define CS_STALL_SEGMENT 1
 #define CS_STALL_SUM 2
 #define CS_STALL_PLAIN 4
+#define CS_STALL_CODES 5
 cs_status cs_test_wait(cs_ctx* ctx, int64_t limit_ns, int stall);
 
 /*

@@ -37,6 +37,7 @@ STALL_NONE = 0
 STALL_SEGMENT = 1
 STALL_SUM = 2
 STALL_PLAIN = 4
+STALL_CODES = 5
 
 # every symbol include/cosparse.h declares
 EXPORTS = (

@@ -412,7 +412,8 @@ cs_status cs_refined_count(cs_ctx* ctx, int32_t* count, void* stream) {
 cs_status cs_test_wait(cs_ctx* ctx, int64_t limit_ns, int stall) {
     if (!ctx) return cs_set_error(nullptr, CS_ERR_INVALID_ARG, "cs_test_wait: ctx is NULL");
     if (limit_ns < 0 || (stall != CS_STALL_NONE && stall != CS_STALL_SEGMENT &&
-                         stall != CS_STALL_SUM && stall != CS_STALL_PLAIN))
+                         stall != CS_STALL_SUM && stall != CS_STALL_PLAIN &&
+                         stall != CS_STALL_CODES))
         return cs_set_error(ctx, CS_ERR_INVALID_ARG, "cs_test_wait: limit %lld ns, stall %d",
                             (long long)limit_ns, stall);
     ctx->wait_ns = (unsigned long long)limit_ns;
@@ -606,8 +607,11 @@ void cs_lik_carve(Carve& c, LikPlan& L, int32_t* dist2) {
     L.flags = c.take<unsigned long long>(L.tc_form ? (size_t)P : 0);
 }
 
-static cudaError_t enqueue_codes(cs_ctx* ctx, const CodesArgs& a, cudaStream_t st) {
+static cudaError_t enqueue_codes(cs_ctx* ctx, CodesArgs a, cudaStream_t st) {
     StageTimer tm(ctx, CS_STAGE_CODES, st);
+    a.wait_ns = ctx->wait_ns;
+    a.stall = a.tc && ctx->stall == CS_STALL_CODES;  // the timeout-path test hook, one-shot
+    if (a.stall) ctx->stall = CS_STALL_NONE;
     return launch_codes(a, st);
 }
 

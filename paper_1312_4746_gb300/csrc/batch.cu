@@ -158,7 +158,11 @@ static cudaError_t enqueue_run(cs_batch* b, cudaStream_t st) {
                        L.vbuf, L.fbuf, L.d2, ctx->d_err};
             e = launch_edt(ea, ss);
         }
-        if (e == cudaSuccess && !b->codes_given) e = launch_codes(m.codes, ss);
+        if (e == cudaSuccess && !b->codes_given) {
+            CodesArgs ca = m.codes;
+            ca.wait_ns = ctx->wait_ns;
+            e = launch_codes(ca, ss);
+        }
         if (e == cudaSuccess && b->prm.mode == CS_MODE_FACTORISED)
             e = launch_majority(L.H, L.W, m.codes.bitmask, L.k, L.n_labels, L.d_off, m.d.sample_pix,
                                 L.t.rep, ss);

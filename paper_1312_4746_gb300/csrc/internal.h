@@ -148,6 +148,9 @@ struct CodesArgs {
     // patch order 1 (centre, mask, centre again, normalise): every code in
     // double precision in the canonical order (no guard list)
     int order = 0;
+    // tensor-core form
+    unsigned long long wait_ns = 0;  // limit of each barrier wait (0: 1 s)
+    bool stall = false;  // timeout-path test: the last block waits for what nothing completes
 };
 // FP32 CUDA-core codes, or (a.tc) the tcgen05 split-BF16 GEMM; both followed
 // by the canonical FP64 recompute of guarded entries.

@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(128) codes_fp64_kernel(
 // closer to tau than the bound go to the same guard list and canonical FP64
 // recompute as the FP32 form.
 constexpr int CT_W = 16, CT_H = 8;  // pixel tile: 128 pixels
-constexpr uint64_t CT_WAIT_NS = 1000000000ull;
+constexpr uint64_t CT_WAIT_NS = 1000000000ull;  // default limit of a wait
 
 __host__ __device__ constexpr int ct_ks(int p) { return (p * p + 15) / 16; }
 __host__ __device__ constexpr int ct_np(int k) { return (k + 15) / 16 * 16; }
@@ -607,14 +607,15 @@ __global__ void __launch_bounds__(128, 4) codes_tc_kernel(
     const float* __restrict__ mask, const float* __restrict__ rownorm, float tau_f,
     float tau_slack, float* __restrict__ codes, float* __restrict__ lead16,
     uint32_t* __restrict__ bitmask, int2* __restrict__ guard, int guard_cap,
-    int* __restrict__ guard_count, int* __restrict__ d_err) {
+    int* __restrict__ guard_count, int* __restrict__ d_err, uint64_t wait_ns, bool stall) {
     constexpr int N = P * P, R = (P - 1) / 2, KS = ct_ks(P);
     constexpr int GW = CT_W + P - 1, GH = CT_H + P - 1;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* sa = smem;                                  // A: 3 KS slabs x 4096 B
     uint8_t* sb = smem + 3 * KS * 4096;                  // B: 3 KS slabs x np x 32 B
     uint8_t* misc = sb + 3 * KS * np * 32;               // 32-byte aligned
-    uint64_t* bars = reinterpret_cast<uint64_t*>(misc);  // [0] B copy, [1] MMA
+    // [0] B copy, [1] MMA, [3] nothing (the timeout-path test)
+    uint64_t* bars = reinterpret_cast<uint64_t*>(misc);
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(misc + 16);
     int* s_flag = reinterpret_cast<int*>(misc + 20);
     float* s_gray = reinterpret_cast<float*>(misc + 32);
@@ -628,6 +629,7 @@ __global__ void __launch_bounds__(128, 4) codes_tc_kernel(
     if (tid == 0) {
         tc::mbar_init(bars + 0, 1);
         tc::mbar_init(bars + 1, 1);
+        tc::mbar_init(bars + 3, 1);
         tc::fence_mbar_init();
         tc::mbar_arrive_expect_tx(bars + 0, b_bytes);
         tc::bulk_g2s(sb, blob, b_bytes, bars + 0);
@@ -735,7 +737,10 @@ __global__ void __launch_bounds__(128, 4) codes_tc_kernel(
     // ---- MMA (one thread) ---------------------------------------------------
     if (tid == 0) {
         int flag = 0;
-        if (tc::mbar_wait(bars + 0, 0, tc::globaltimer() + CT_WAIT_NS)) {
+        // (the timeout-path test: the last block waits for what nothing completes)
+        const bool go = !(stall && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1) ||
+                        tc::mbar_wait(bars + 3, 0, tc::globaltimer() + wait_ns);
+        if (go && tc::mbar_wait(bars + 0, 0, tc::globaltimer() + wait_ns)) {
             tc::fence_after_sync();
             const uint32_t id = tc::idesc(128, np, 1, 1);
             // (operator piece, patch piece), smallest products first
@@ -752,13 +757,13 @@ __global__ void __launch_bounds__(128, 4) codes_tc_kernel(
         } else {
             ct_set_error(d_err, 21);
             // the copy must land before the CTA may exit
-            tc::mbar_wait(bars + 0, 0, tc::globaltimer() + CT_WAIT_NS);
+            tc::mbar_wait(bars + 0, 0, tc::globaltimer() + wait_ns);
         }
         *s_flag = flag;
     }
     __syncthreads();
     bool ok = *s_flag != 0;
-    if (ok && !tc::mbar_wait(bars + 1, 0, tc::globaltimer() + CT_WAIT_NS)) {
+    if (ok && !tc::mbar_wait(bars + 1, 0, tc::globaltimer() + wait_ns)) {
         ok = false;
         ct_set_error(d_err, 22);
     }
@@ -788,7 +793,7 @@ __global__ void __launch_bounds__(128, 4) codes_tc_kernel(
         if (live && whole) guard_push(guard, guard_cap, guard_count, pix, -1);
     } else if (tid == 0 && *s_flag) {
         // MMAs still in flight: they must finish before the tensor memory is freed
-        tc::mbar_wait(bars + 1, 0, tc::globaltimer() + CT_WAIT_NS);
+        tc::mbar_wait(bars + 1, 0, tc::globaltimer() + wait_ns);
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -832,11 +837,11 @@ __host__ __device__ constexpr CpOff cp_off(int np) {
     return o;
 }
 
-// Bounded wait shared by the roles: gives up after CT_WAIT_NS or once
+// Bounded wait shared by the roles: gives up after wait_ns or once
 // another role has aborted.
 __device__ __forceinline__ bool cp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                        int* d_err, int site) {
-    const uint64_t deadline = tc::globaltimer() + CT_WAIT_NS;
+                                        int* d_err, int site, uint64_t wait_ns) {
+    const uint64_t deadline = tc::globaltimer() + wait_ns;
     for (uint32_t n = 0;; ++n) {
         if (tc::mbar_try_wait(bar, parity, 1000u)) return true;
         if ((n & 63u) == 63u && (*abort_flag || tc::globaltimer() > deadline)) break;
@@ -849,8 +854,9 @@ __device__ __forceinline__ bool cp_wait(uint64_t* bar, uint32_t parity, volatile
 // The same by a whole warp, with one outcome: lanes on either side of the deadline
 // would part before the barriers and warp-wide loads that follow.
 __device__ __forceinline__ bool cp_wait_warp(uint64_t* bar, uint32_t parity,
-                                             volatile int* abort_flag, int* d_err, int site) {
-    return __all_sync(0xffffffffu, cp_wait(bar, parity, abort_flag, d_err, site));
+                                             volatile int* abort_flag, int* d_err, int site,
+                                             uint64_t wait_ns) {
+    return __all_sync(0xffffffffu, cp_wait(bar, parity, abort_flag, d_err, site, wait_ns));
 }
 
 template <int P>
@@ -859,7 +865,7 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
     const float* __restrict__ mask, const float* __restrict__ rownorm, float tau_f,
     float tau_slack, float* __restrict__ codes, float* __restrict__ lead16,
     uint32_t* __restrict__ bitmask, int2* __restrict__ guard, int guard_cap,
-    int* __restrict__ guard_count, int* __restrict__ d_err) {
+    int* __restrict__ guard_count, int* __restrict__ d_err, uint64_t wait_ns, bool stall) {
     constexpr int N = P * P, R = (P - 1) / 2, KS = ct_ks(P);
     constexpr int WW = CT_W + P - 1, WH = P + 1;
     constexpr int EG = cp_groups(P), NTHR = cp_threads(P), MMA_WARP = 4 + 4 * EG;
@@ -890,6 +896,7 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
         tc::mbar_init(b_full, 1);
         tc::mbar_init(a_full, 4);
         tc::mbar_init(a_empty, 1);
+        tc::mbar_init(bars + 11, 1);
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(t_full + b, 1);
             tc::mbar_init(t_empty + b, 4 * EG);
@@ -970,7 +977,7 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
                                      5 * KS * 4.76837158203125e-07f * 0.0079f;
             const float ebase = (ds + EPS_TC * (1.f + ds)) * 1.25f;
             // the A operand is free once the previous tile's MMAs have read it
-            if (!cp_wait_warp(a_empty, (uint32_t)((kk & 1) ^ 1), abort_flag, d_err, 23)) break;
+            if (!cp_wait_warp(a_empty, (uint32_t)((kk & 1) ^ 1), abort_flag, d_err, 23, wait_ns)) break;
 #pragma unroll
             for (int sl = 0; sl < KS; ++sl) {
                 uint32_t w1[8], w2[8], w3[8];
@@ -1013,7 +1020,9 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
             if (lane == 0) tc::mbar_arrive(a_full);
             // this pixel's parameters for the epilogue
             const int pb = kk & 1;
-            if (!cp_wait_warp(p_empty + pb, (uint32_t)(((kk >> 1) & 1) ^ 1), abort_flag, d_err, 24)) break;
+            if (!cp_wait_warp(p_empty + pb, (uint32_t)(((kk >> 1) & 1) ^ 1), abort_flag, d_err, 24,
+                              wait_ns))
+                break;
             prm[pb * 128 + r] = make_int4(live ? pix : -1, whole ? 1 : 0, __float_as_int(ebase), 0);
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(p_full + pb);
@@ -1026,11 +1035,13 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
         int kk = 0;
         for (int T = blockIdx.x; T < ntiles; T += gridDim.x, ++kk) {
             const int b = kk & 1;
-            if (!cp_wait_warp(p_full + b, (uint32_t)((kk >> 1) & 1), abort_flag, d_err, 25)) break;
+            if (!cp_wait_warp(p_full + b, (uint32_t)((kk >> 1) & 1), abort_flag, d_err, 25, wait_ns))
+                break;
             const int4 pp = prm[b * 128 + 32 * q + lane];
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(p_empty + b);
-            if (!cp_wait_warp(t_full + b, (uint32_t)((kk >> 1) & 1), abort_flag, d_err, 26)) break;
+            if (!cp_wait_warp(t_full + b, (uint32_t)((kk >> 1) & 1), abort_flag, d_err, 26, wait_ns))
+                break;
             tc::fence_after_sync();
             const bool live = pp.x >= 0, whole = pp.y != 0;
             const int pix = live ? pp.x : 0;
@@ -1060,13 +1071,18 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
     } else if (lane == 0) {
         // ---------------------------------------------------------- MMA issuer
         long long last = -1;
-        if (cp_wait(b_full, 0, abort_flag, d_err, 21)) {
+        // (the timeout-path test: the last block waits for what nothing completes,
+        // before it issues anything)
+        const bool go = !(stall && blockIdx.x == gridDim.x - 1) ||
+                        cp_wait(bars + 11, 0, abort_flag, d_err, 20, wait_ns);
+        if (go && cp_wait(b_full, 0, abort_flag, d_err, 21, wait_ns)) {
             const uint32_t id = tc::idesc(128, np, 1, 1);
             int kk = 0;
             for (int T = blockIdx.x; T < ntiles; T += gridDim.x, ++kk) {
                 const int b = kk & 1;
-                if (!cp_wait(a_full, (uint32_t)(kk & 1), abort_flag, d_err, 22) ||
-                    !cp_wait(t_empty + b, (uint32_t)(((kk >> 1) & 1) ^ 1), abort_flag, d_err, 27))
+                if (!cp_wait(a_full, (uint32_t)(kk & 1), abort_flag, d_err, 22, wait_ns) ||
+                    !cp_wait(t_empty + b, (uint32_t)(((kk >> 1) & 1) ^ 1), abort_flag, d_err, 27,
+                             wait_ns))
                     break;
                 tc::fence_after_sync();
                 const uint32_t d = tmem + (uint32_t)(b * ncols);
@@ -1085,12 +1101,12 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
             }
         } else {
             // the copy must land before the CTA may exit
-            tc::mbar_wait(b_full, 0, tc::globaltimer() + CT_WAIT_NS);
+            tc::mbar_wait(b_full, 0, tc::globaltimer() + wait_ns);
         }
         // drain: the last MMAs must finish before the tensor memory is freed
         if (last >= 0)
             tc::mbar_wait(t_full + (int)(last & 1), (uint32_t)((last >> 1) & 1),
-                          tc::globaltimer() + CT_WAIT_NS);
+                          tc::globaltimer() + wait_ns);
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -1117,6 +1133,7 @@ size_t ct_smem(int np) {
 template <int P>
 cudaError_t launch_tc_p(const CodesArgs& a, cudaStream_t st) {
     const int np = ct_np(a.k);
+    const uint64_t wait_ns = a.wait_ns ? a.wait_ns : CT_WAIT_NS;
     const size_t smem = ct_smem<P>(np);
     cudaError_t e = cs_smem_limit((const void*)codes_tc_kernel<P>, ct_smem<P>(256));
     if (e != cudaSuccess) return e;
@@ -1138,7 +1155,7 @@ cudaError_t launch_tc_p(const CodesArgs& a, cudaStream_t st) {
         codes_tc_kernel<P><<<grd, 128, smem, st>>>(a.img, a.H, a.W, a.omega_blob, a.k, np, a.mask,
                                                    a.rownorm, tau_f, slack, a.codes, a.lead16,
                                                    a.bitmask, a.guard, a.guard_cap, a.guard_count,
-                                                   a.d_err);
+                                                   a.d_err, wait_ns, a.stall);
         return cudaGetLastError();
     }
     const size_t floor_b = 233472 / (per_sm + 1) - 1024 + 16;  // no further CTA fits
@@ -1153,7 +1170,7 @@ cudaError_t launch_tc_p(const CodesArgs& a, cudaStream_t st) {
     const int grid = ntiles < per_sm * n_sm ? ntiles : per_sm * n_sm;
     codes_tcp_kernel<P><<<grid, cp_threads(P), psmem, st>>>(
         a.img, a.H, a.W, a.omega_blob, a.k, np, a.mask, a.rownorm, tau_f, slack, a.codes,
-        a.lead16, a.bitmask, a.guard, a.guard_cap, a.guard_count, a.d_err);
+        a.lead16, a.bitmask, a.guard, a.guard_cap, a.guard_count, a.d_err, wait_ns, a.stall);
     return cudaGetLastError();
 }
 

@@ -1,7 +1,8 @@
 """The give-up path of the bounded waits in the forms that test_gpu_timeout.py's
 calls do not reach: the solver's tile form with a label cost (which also waits for
-the blocks' sums) and its general form (grid barriers; more than 16 labels), and the
-plain FP32 sum's wait for its tensor-core products. As there: the one-shot hook makes
+the blocks' sums) and its general form (grid barriers; more than 16 labels), the plain
+FP32 sum's wait for its tensor-core products, and the tensor-core codes (pipelined,
+and the kernel for operators too large for that). As there: the one-shot hook makes
 one wait run out before anything is in flight, the call reports the timeout within
 the shortened limit, and the next call gives the earlier bits.
 """
@@ -79,6 +80,31 @@ def test_plain_sum(env, H, W):
     ctx.test_wait(LIMIT_NS, cs.STALL_PLAIN)
     call(cs.Params.from_synth(pr.params, mode=cs.MODE_FACTORISED))
     call(cs.Params.from_synth(pr.params, precision=cs.FP8))
+    ctx.sync()
+    ctx.test_wait(0, cs.STALL_NONE)
+    assert torch.equal(call(), ref)
+    ctx.sync()
+
+
+@pytest.mark.parametrize("p,k", [(5, 50), (9, 98), (9, 256)])
+def test_codes(env, p, k):
+    cs, ctx, torch = env
+    pr = synth.make_problem(64, 96, 2, 20, p=p, k=k, seed=78)
+    img, om, mask = (torch.from_numpy(np.ascontiguousarray(a)).to("cuda:0")
+                     for a in (pr.image, pr.omega, pr.mask))
+    prm = cs.Params.from_synth(pr.params, codes_form=cs.CODES_TC)
+
+    def call(q=prm):
+        return ctx.codes(img, om, mask, q)["bitmask"]
+
+    ref = call()
+    ctx.sync()
+    # the first wait to give up records its site: the stalled one or one that
+    # depends on it
+    assert 20 <= _stalled(cs, ctx, cs.STALL_CODES, call) <= 27
+    assert torch.equal(call(), ref)
+    ctx.test_wait(LIMIT_NS, cs.STALL_CODES)  # a form without that wait leaves it armed
+    assert torch.equal(call(cs.Params.from_synth(pr.params, codes_form=cs.CODES_FP32)), ref)
     ctx.sync()
     ctx.test_wait(0, cs.STALL_NONE)
     assert torch.equal(call(), ref)
