@@ -272,7 +272,8 @@ cs_status cs_cosupport(cs_ctx* ctx, const float* codes, int P, int k, double tau
  * the majority co-support of the label's samples (Eq. tex-rep).
  *
  *   img        DEVICE H x W x 3 float32
- *   bitmask    DEVICE P x ceil(k/32) uint32 (from cs_codes)
+ *   bitmask    DEVICE P x ceil(k/32) uint32 (from cs_codes; the last word's bits
+ *              beyond the k codes are ignored)
  *   label_off  HOST   n_labels + 1 int32, CSR offsets into sample_pix;
  *              label_off[0] = 0 and every label needs >= 1 sample
  *   sample_pix DEVICE label_off[n_labels] int32 pixel indices (y*W + x)

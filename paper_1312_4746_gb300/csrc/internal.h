@@ -113,6 +113,13 @@ cs_status cs_set_error(cs_ctx* ctx, cs_status code, const char* fmt, ...);
 cs_status cs_ensure_scratch(cs_ctx* ctx, size_t bytes);
 cs_status cs_check_launch(cs_ctx* ctx, const char* what);
 
+// Bits of word w of a co-support bitmask that are codes below k. A caller's bitmask
+// may hold anything in the others: the texture similarity is over the k codes.
+__host__ __device__ inline uint32_t code_mask(int w, int k) {
+    const int left = k - 32 * w;
+    return left >= 32 ? 0xffffffffu : left > 0 ? (1u << left) - 1u : 0u;
+}
+
 // Dynamic shared memory limit of a kernel, before its launches. The limit belongs to
 // the kernel on the device, not to a launch or a context: `most` is the largest that
 // any call needs, so that a call cannot lower the limit between another thread's
@@ -545,7 +552,7 @@ struct SurrogateEvalArgs {
     const int32_t* label_off;
     const uint32_t* bitmask;
     const uint32_t* rep;
-    int Wk, mode, rule;
+    int k, mode, rule;
     float alpha, d_min, kappa_beta, sigma_c2, margin, eps;
     bool rho_var;
     float* neglog;

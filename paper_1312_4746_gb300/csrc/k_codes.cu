@@ -73,10 +73,6 @@ __device__ __forceinline__ void threshold16(const uint32_t (&v)[16], int sh, con
     word |= w << sh;
     gword |= g << sh;
 }
-// bits of word w that are codes below k
-__device__ __forceinline__ uint32_t word_mask(int w, int k) {
-    return k - 32 * w >= 32 ? 0xffffffffu : (1u << (k - 32 * w)) - 1u;
-}
 
 // the guard entries of one 32-code word
 __device__ __forceinline__ void guard_word(int2* guard, int cap, int* count, int pix, int w,
@@ -782,7 +778,7 @@ __global__ void __launch_bounds__(128, 4) codes_tc_kernel(
             threshold16(v, 16 * (c & 1), s_rn + 16 * c, ebase, tau_f, tau_slack, word, gword);
             store_codes(v, c, live, pix, k, codes, lead16);
             if ((c & 1) || c == np / 16 - 1) {
-                const uint32_t m = word_mask(c >> 1, k);
+                const uint32_t m = code_mask(c >> 1, k);
                 word &= m;
                 gword &= m;
                 if (live && !whole) guard_word(guard, guard_cap, guard_count, pix, c >> 1, gword);
@@ -1059,7 +1055,7 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
                         store_codes(v, c, live, pix, k, codes, lead16);
                     }
                 }
-                const uint32_t m = word_mask(wd, k);
+                const uint32_t m = code_mask(wd, k);
                 if (live && !whole) guard_word(guard, guard_cap, guard_count, pix, wd, gword & m);
                 if (live && bitmask) bitmask[(size_t)pix * Wk + wd] = whole ? 0u : word & m;
             }

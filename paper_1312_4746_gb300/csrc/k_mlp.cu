@@ -614,7 +614,7 @@ struct FwdArgs {
     const int32_t* label_off;
     const uint32_t* bitmask;
     const uint32_t* rep;
-    int Wk, mode, rule;
+    int k, Wk, mode, rule;
     float alpha, kappa_beta, sigma_c2, margin, eps;
     bool rho_var;
     float* neglog;
@@ -651,7 +651,9 @@ __device__ void eval_pixel(const FwdArgs& a, long long q, float (&z)[64], const 
     const float log_col_norm = 1.5f * logf(6.283185307179586f * a.sigma_c2);
     uint32_t bx[8];
     for (int w = 0; w < 8; ++w)
-        bx[w] = (a.mode == CS_MODE_FACTORISED && w < a.Wk) ? a.bitmask[q * a.Wk + w] : 0u;
+        bx[w] = (a.mode == CS_MODE_FACTORISED && w < a.Wk)
+                    ? a.bitmask[q * a.Wk + w] & code_mask(w, a.k)
+                    : 0u;
     float tmax = -INFINITY;
     float tex[64];  // factorised mode: the texture exponents -h_j / beta_j
     for (int j = 0; j < n; ++j) {
@@ -1017,7 +1019,8 @@ cudaError_t launch_surrogate_eval(const SurrogateEvalArgs& s, cudaStream_t st) {
     a.label_off = s.label_off;
     a.bitmask = s.bitmask;
     a.rep = s.rep;
-    a.Wk = s.Wk;
+    a.k = s.k;
+    a.Wk = (s.k + 31) / 32;
     a.mode = s.mode;
     a.rule = s.rule;
     a.alpha = s.alpha;

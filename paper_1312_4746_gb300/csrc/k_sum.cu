@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(256) plain_tiles_kernel(
 #pragma unroll
     for (int c = 0; c < 3; ++c) f[(2 + c) * TS + r] = ok ? img[(size_t)pix * 3 + c] : 0.f;
     for (int w = 0; w < KS; ++w) {
-        uint32_t bits = ok && w < Wk ? bitmask[(size_t)pix * Wk + w] : 0u;
+        uint32_t bits = ok && w < Wk ? bitmask[(size_t)pix * Wk + w] & code_mask(w, k) : 0u;
         for (int c = k; c < k + 2; ++c)  // the columns of -|b_x|
             if (c >> 5 == w) bits |= 1u << (c & 31);
         uint8_t* slab = base + 5 * TS * 4 + w * TS * 32;
@@ -259,18 +259,18 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
         // operand row of pixel tid (PT = 1: the first 128 threads)
         if (TEX && tid < BP) {
             const uint32_t* bx = a.bitmask + pixel_of(item0 + tid) * a.Wk;
-            int pop = 0;
+            int pop = -__popc(bx[a.Wk - 1] & ~code_mask(a.Wk - 1, a.k));  // (bits that are no codes)
             for (int w = 0; w < a.Wk; ++w) pop += __popc(bx[w]);
             const uint32_t hi = e4m3_minus(pop & ~15), lo = e4m3_minus(pop & 15);
 #pragma unroll
             for (int w = 0; w < KS; ++w) {
                 const int left = a.k - 32 * w;  // codes from this step on
+                const uint32_t valid = code_mask(w, a.k);
                 const uint32_t bits = left > 0 ? bx[w] : 0u;
-                const uint32_t valid = left >= 32 ? ~0u : left > 0 ? (1u << left) - 1u : 0u;
                 uint32_t v[8];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
-                    v[q] = spread((bits >> (4 * q)) & 15u, E4M3_ONE) |
+                    v[q] = spread(((bits & valid) >> (4 * q)) & 15u, E4M3_ONE) |
                            spread(((~bits & valid) >> (4 * q)) & 15u, E4M3_MINUS);
                     const int c0 = left - 4 * q, c1 = c0 + 1;  // the columns of -|b_x|
                     if (c0 >= 0 && c0 < 4) v[q] |= hi << (8 * c0);
@@ -479,11 +479,12 @@ __global__ void __launch_bounds__(256) normalise_plain_kernel(SumArgs a) {
         const long long q = a.pix_list ? (long long)a.pix_list[it] : it;
         if (a.mode == CS_MODE_FACTORISED) {
             const uint32_t* bx = a.bitmask + (size_t)q * a.Wk;
+            const int pad = __popc(bx[a.Wk - 1] & ~code_mask(a.Wk - 1, a.k));  // bits that are no codes
             auto logit = [&](int i) {
                 float rho, nA, nB;
                 label_consts(a.dist2[(size_t)i * P + q], a.alpha, a.d_min, a.kappa_beta, a.rho_var,
                              rho, nA, nB);
-                int h = 0;
+                int h = -pad;
                 for (int w = 0; w < a.Wk; ++w) h += __popc(bx[w] ^ a.t.rep[i * a.Wk + w]);
                 return nB * (float)h;
             };

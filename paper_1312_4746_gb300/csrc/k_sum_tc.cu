@@ -465,9 +465,10 @@ __device__ void normalise_pixel(const TcArgs& a, const TcImage& im, int pix, con
     const long long P = (long long)im.H * im.W;
     float* nl = im.neglog + pix;
     if (!PERSAMPLE && im.rep) {  // factorised: the majority-co-support posterior
+        const int pad = __popc(bxp[a.Wk - 1] & ~code_mask(a.Wk - 1, a.k));  // bits that are no codes
         auto logit = [&](int i) {
             const float rho = a.alpha * fmaxf(sqrtf((float)im.dist2[(size_t)i * P + pix]), a.d_min);
-            int h = 0;
+            int h = -pad;
             for (int w = 0; w < a.Wk; ++w) h += __popc(bxp[w] ^ im.rep[i * a.Wk + w]);
             return -LOG2E * (float)h / (a.kappa_beta * rho);
         };
@@ -850,7 +851,10 @@ __global__ void __launch_bounds__((Cfg<TEX8, KS, PERSAMPLE, SOLO>::THREADS),
             p.I2 = fmaf(p.IR, p.IR, fmaf(p.IG, p.IG, p.IB * p.IB));
             p.popx = 0;
 #pragma unroll
-            for (int w = 0; w < WKM; ++w) p.popx += p.live ? __popc(p.bw[w]) : 0;
+            for (int w = 0; w < WKM; ++w) {
+                p.bw[w] &= code_mask(w, a.k);  // (0 beyond the last word)
+                p.popx += p.live ? __popc(p.bw[w]) : 0;
+            }
         };
         // texture operand rows of a pixel tile (the codes of the MMA slabs):
         // this warp writes slabs sl = hf, hf + EPQ, ... of buffer pwr % ATB
@@ -1172,7 +1176,7 @@ __global__ void __launch_bounds__((Cfg<TEX8, KS, PERSAMPLE, SOLO>::THREADS),
 // double for the pixel.
 __global__ void __launch_bounds__(128) refine_fp64_kernel(
     const TcImage* __restrict__ images, const int4* __restrict__ list,
-    const int* __restrict__ count, int cap, const unsigned long long* __restrict__ flags, int Wk,
+    const int* __restrict__ count, int cap, const unsigned long long* __restrict__ flags, int k,
     double alpha, double d_min, double kappa_beta, double sigma_c2, bool persample, bool rho_var,
     int* __restrict__ d_err) {
     __shared__ double sL[4][CS_MAX_LABELS];
@@ -1183,7 +1187,7 @@ __global__ void __launch_bounds__(128) refine_fp64_kernel(
             d_err[1] = cnt;
         cnt = cap;
     }
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, Wk = (k + 31) / 32;
     const int nwarps = gridDim.x * 4;
     const double PI2 = 6.283185307179586;
     const double col_norm = 1.5 * log(PI2 * sigma_c2), c_col = 0.5 / sigma_c2;
@@ -1197,7 +1201,8 @@ __global__ void __launch_bounds__(128) refine_fp64_kernel(
                      IB = im.img[(size_t)pix * 3 + 2];
         uint32_t bx[8];
 #pragma unroll
-        for (int w = 0; w < 8; ++w) bx[w] = w < Wk ? im.bitmask[(size_t)pix * Wk + w] : 0u;
+        for (int w = 0; w < 8; ++w)
+            bx[w] = w < Wk ? im.bitmask[(size_t)pix * Wk + w] & code_mask(w, k) : 0u;
         for (int i = 0; i < im.n_labels; ++i) {
             const double rho = alpha * fmax(sqrt((double)im.dist2[(size_t)i * P + pix]), d_min);
             if (lane == 0 && !persample && im.rep) {
@@ -1382,7 +1387,7 @@ __global__ void __launch_bounds__(BN) build_tiles_kernel(
     uint32_t bits[WMAX];
 #pragma unroll
     for (int w = 0; w < WMAX; ++w)
-        bits[w] = valid && w < Wk ? bitmask[(size_t)pix * Wk + w] : 0u;
+        bits[w] = valid && w < Wk ? bitmask[(size_t)pix * Wk + w] & code_mask(w, k) : 0u;
     const float R = img[(size_t)pix * 3], G = img[(size_t)pix * 3 + 1], B = img[(size_t)pix * 3 + 2];
     const int x = pix % W, y = pix / W;
     if (valid) {
@@ -1534,8 +1539,8 @@ cudaError_t sum(const TcImage* descs, int n_images, const TcSumParams& p, cudaSt
     a.i1 = i1;
     sum_tc_kernel<TEX8, KS, PERSAMPLE, SOLO><<<grid, C::THREADS, C::smem_bytes, st>>>(a);
     refine_fp64_kernel<<<2 * p.n_sm, 128, 0, st>>>(
-        descs, p.fb_list, p.fb_count, p.fb_cap, p.flags, (p.k + 31) / 32, (double)p.alpha,
-        (double)p.d_min, (double)p.kappa_beta, (double)p.sigma_c2, PERSAMPLE, p.rho_var, p.d_err);
+        descs, p.fb_list, p.fb_count, p.fb_cap, p.flags, p.k, (double)p.alpha, (double)p.d_min,
+        (double)p.kappa_beta, (double)p.sigma_c2, PERSAMPLE, p.rho_var, p.d_err);
     const long long nblk = (p.total_pixels + 255) / 256, cap = 8ll * p.n_sm;
     normalise_kernel<PERSAMPLE><<<(unsigned)(nblk < cap ? nblk : cap), 256, 0, st>>>(a);
     return cudaGetLastError();

@@ -317,7 +317,7 @@ cs_status cs_surrogate_eval(cs_ctx* ctx, const float* img, int H, int W, const u
         a.label_off = cs_plan_label_off(plan);
         a.bitmask = bitmask;
         a.rep = cs_plan_rep(plan);
-        a.Wk = (k + 31) / 32;
+        a.k = k;
         a.mode = prm->mode;
         a.alpha = (float)prm->alpha;
         a.d_min = (float)prm->d_min;
