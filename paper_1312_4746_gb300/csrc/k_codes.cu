@@ -575,19 +575,20 @@ __device__ __forceinline__ void ct_set_error(int* d_err, int site) {
 }
 
 // The 16 codes of chunk c to the callers' arrays: `codes` (k per pixel), and the
-// first chunk to `lead16` (zero beyond k: the operator's padding rows are zero).
+// first chunk to `lead16` (zero beyond k, also where a patch holds a NaN or infinity,
+// whose products with the operator's zero padding rows are NaN).
 __device__ __forceinline__ void store_codes(const uint32_t (&v)[16], int c, bool live, int pix, int k,
                                             float* __restrict__ codes, float* __restrict__ lead16) {
     if (lead16 && c == 0 && live) {
         float4* d = reinterpret_cast<float4*>(lead16 + (size_t)pix * 16);
+        auto code = [&](int e) { return e < k ? __uint_as_float(v[e]) : 0.f; };
         if ((reinterpret_cast<uintptr_t>(d) & 15) == 0) {
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                d[q] = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
-                                   __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
+                d[q] = make_float4(code(4 * q), code(4 * q + 1), code(4 * q + 2), code(4 * q + 3));
         } else {
 #pragma unroll
-            for (int e = 0; e < 16; ++e) lead16[(size_t)pix * 16 + e] = __uint_as_float(v[e]);
+            for (int e = 0; e < 16; ++e) lead16[(size_t)pix * 16 + e] = code(e);
         }
     }
     if (codes && live) {
