@@ -584,21 +584,22 @@ void cs_lik_carve(Carve& c, LikPlan& L, int32_t* dist2) {
     L.d_off = c.take<int32_t>(2 * (n + 1));
     L.seedbits = c.take<uint32_t>((size_t)n * L.H * ((L.W + 31) / 32));
     L.colbuf = c.take<int32_t>(P * n);
-    // envelope stacks: two halves of (H + 1) / 2 rows per column
+    // envelope stacks
     L.vbuf = c.take<int32_t>((size_t)(L.H + 7) * L.W * n);  // S ceil(H / S) <= H + 7 rows
     L.fbuf = c.take<int32_t>((size_t)(L.H + 7) * L.W * n);
     int32_t* d2s = c.take<int32_t>(dist2 ? 0 : P * n);
     L.d2 = dist2 ? dist2 : d2s;
-    L.t.sx = c.take<float>(S);
-    L.t.sy = c.take<float>(S);
-    L.t.sr = c.take<float>(S);
-    L.t.sg = c.take<float>(S);
-    L.t.sb = c.take<float>(S);
-    L.t.sbits = c.take<uint32_t>((size_t)Wk * S);
+    const size_t St = L.tc_form ? (size_t)S : 0;  // the plain form reads its tiles only
+    L.t.sx = c.take<float>(St);
+    L.t.sy = c.take<float>(St);
+    L.t.sr = c.take<float>(St);
+    L.t.sg = c.take<float>(St);
+    L.t.sb = c.take<float>(St);
+    L.t.sbits = c.take<uint32_t>(Wk * St);
     L.t.rep = c.take<uint32_t>((size_t)n * Wk);
     L.t.blob = c.take<uint8_t>((size_t)L.total_tiles * L.stage_bytes, 1024);
     L.t.tile_xy = c.take<uint32_t>(L.tc_form ? (size_t)L.total_tiles * tc_tile_samples() : 0);
-    L.t.perm = c.take<int32_t>(L.tc_form ? (size_t)S : 0);
+    L.t.perm = c.take<int32_t>(St);
     L.desc = c.take<TcImage>(L.tc_form ? 1 : 0);
     L.imax2 = c.take<float>(L.tc_form ? (size_t)n : 0);
     L.fb_list = c.take<int4>(L.tc_form ? (size_t)P : 0);
