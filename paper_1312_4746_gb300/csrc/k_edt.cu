@@ -6,8 +6,8 @@
 //   1. seed bitmaps: one bit per pixel and label;
 //   2. row pass (one warp per label and row): horizontal distance h to the
 //      nearest seed in the same row, from bit scans of the bitmap words;
-//   3. column pass (2, 4 or 8 builder threads per label and column, one per
-//      row segment, and 32 readers): lower envelopes of the parabolas
+//   3. column pass (2 to 6 builder threads per label and column, one per
+//      row segment, and 8 to 32 readers): lower envelopes of the parabolas
 //      (y - q)^2 + h(q)^2 over each segment's rows q with finite h, each
 //      built in one sweep and read back by row ranges; intersection
 //      abscissae are compared as exact rationals with 64-bit cross products,
@@ -97,13 +97,11 @@ __global__ void rows_binary_kernel(int H, int W, int n_labels, const uint32_t* _
 // monotone in the segment index), walks on, and keeps the smallest of the S
 // values, the minimum over all rows.
 //
-// Bound: the sweeps' and the reads' latency: about 0.2 us a row swept and 0.13 us
-// a row and envelope read. Few columns per block give many readers (H / 32 rows
-// each) and blocks for every SM, and with them more segments pay. Measured at
-// 481 x 321, 5 labels: 28 us, against 42 us with 32 columns per block, 4
-// segments and 8 readers (and 54 us with 8 segments).
-constexpr int CB = 8;          // columns per block
-constexpr int NRD = 256 / CB;  // reader threads per column
+// Bound with few columns (labels x width): the sweeps' and the reads' latency,
+// about 0.2 us a row swept and 0.13 us a row and envelope read. Few columns per
+// block give many readers (H / 32 rows each) and blocks for every SM, and with them
+// more segments pay. With many columns: the loads and the reads of each envelope, so
+// that 32 columns per block (whole lines of h and of the result) and few segments do.
 
 __device__ __forceinline__ int env_build(const int32_t* __restrict__ col, int W, int q_lo, int q_hi,
                                          int32_t* v, int32_t* F, long long stride) {
@@ -168,10 +166,11 @@ __device__ __forceinline__ int32_t env_value(EnvCursor& c, const int32_t* v, con
     return (y - c.vj) * (y - c.vj) + (c.Fj - c.vj * c.vj);
 }
 
-template <bool SHARED, int S>
+template <bool SHARED, int S, int CB>  // CB columns per block
 __global__ void __launch_bounds__(256) cols_envelope_split_kernel(
     int H, int W, int n_labels, const int32_t* __restrict__ h, int32_t* __restrict__ gv,
     int32_t* __restrict__ gF, int32_t* __restrict__ dist2) {
+    constexpr int NRD = 256 / CB;  // reader threads per column
     static_assert(S >= 1 && S <= NRD, "segments");
     extern __shared__ int32_t smem[];
     __shared__ int s_kk[S][CB];
@@ -339,38 +338,46 @@ cudaError_t launch_edt(const EdtArgs& a, cudaStream_t st) {
         // rows per block: about two blocks per SM, a multiple of the 8 warps
         int rows = (int)std::min<long long>(64, std::max<long long>(8, (long long)cb * a.H / 304));
         rows = (rows + 7) / 8 * 8;
-        cudaError_t e2 = cudaFuncSetAttribute(cols_scan_kernel,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              880 * 128);
+        cudaError_t e2 = cs_smem_limit((const void*)cols_scan_kernel, 880 * 128);
         if (e2 != cudaSuccess) return e2;
         cols_scan_kernel<<<dim3(cb, (a.H + rows - 1) / rows), 256, (size_t)a.H * 128, st>>>(
             a.H, a.W, a.n_labels, rows, a.colbuf, a.dist2);
         return cudaGetLastError();
     }
     // envelopes of CB columns per block (S segments) in shared memory when they fit
-    const unsigned nblk = (unsigned)((ncol + CB - 1) / CB);
-    auto run = [&](auto seg_c) -> cudaError_t {
-        constexpr int S = decltype(seg_c)::value;
+    auto run = [&](auto seg_c, auto cb_c) -> cudaError_t {
+        constexpr int S = decltype(seg_c)::value, CB = decltype(cb_c)::value;
+        const unsigned nblk = (unsigned)((ncol + CB - 1) / CB);
         const size_t smem = (size_t)((a.H + S - 1) / S) * S * 2 * sizeof(int32_t) * CB;
         if (smem <= 110u * 1024u) {
             // (the limit of every size: captured launches of several sizes share it)
-            cudaError_t e2 = cudaFuncSetAttribute(cols_envelope_split_kernel<true, S>,
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  110 * 1024);
+            cudaError_t e2 =
+                cs_smem_limit((const void*)cols_envelope_split_kernel<true, S, CB>, 110 * 1024);
             if (e2 != cudaSuccess) return e2;
-            cols_envelope_split_kernel<true, S><<<nblk, 256, smem, st>>>(
+            cols_envelope_split_kernel<true, S, CB><<<nblk, 256, smem, st>>>(
                 a.H, a.W, a.n_labels, a.colbuf, nullptr, nullptr, a.dist2);
         } else {
-            cols_envelope_split_kernel<false, S><<<nblk, 256, 0, st>>>(
+            cols_envelope_split_kernel<false, S, CB><<<nblk, 256, 0, st>>>(
                 a.H, a.W, a.n_labels, a.colbuf, a.vbuf, a.fbuf, a.dist2);
         }
         return cudaSuccess;
     };
-    // sweeps and reads balance at about 7 segments of H rows; short images have
-    // too few rows for as many
-    e = a.H > 64 ? run(std::integral_constant<int, 8>{})
-      : a.H > 32 ? run(std::integral_constant<int, 4>{})
-                 : run(std::integral_constant<int, 2>{});
+    using std::integral_constant;
+    // Measured, the transform's three launches, us, columns per block / segments:
+    //                  columns   8/6   8/8  16/4  32/2  32/3
+    //   481 x 321 x 5     2405    44    46    50    67    58
+    //   640 x 480 x 5     3200    54    60    65    96    83
+    //   2000 x 200 x 3    6000    42    46    40    42    42
+    //   640 x 480 x 10    6400    86    93    67    95    87
+    //   3000 x 400 x 4   12000   116   129   115   141   128
+    //   481 x 321 x 30   14430    76    88    69    77    78
+    //   2000 x 200 x 8   16000    65    75    55    46    48
+    //   1024 x 1024 x 32 32768   518   639   386   345   321
+    //   23000 x 64 x 2   46000   239   249   218   208   211
+    e = ncol < 6000    ? run(integral_constant<int, 6>{}, integral_constant<int, 8>{})
+        : a.H <= 256   ? run(integral_constant<int, 2>{}, integral_constant<int, 32>{})
+        : ncol < 16000 ? run(integral_constant<int, 4>{}, integral_constant<int, 16>{})
+                       : run(integral_constant<int, 3>{}, integral_constant<int, 32>{});
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
