@@ -228,7 +228,10 @@ __global__ void __launch_bounds__(TILE* TILE)
 // spent five steps and, with a quotient per element and |O_j| and A summed in
 // FP64 too, about 300 warp-wide FP64 operations an entry. Measured at 1023 x 769,
 // 9 x 9 patches, k = 162: 47 us against 128 us; 481 x 321, 7 x 7, k = 98:
-// 10 us against 14 us.
+// 10 us against 14 us. A short list leaves the pipe idle and the chain of a lane's
+// elements counts: up to six entries per SM a whole warp takes one. Measured, the
+// whole codes call, us, eight lanes and 32: 64 x 48, 9 x 9, k = 98: 22.8, 19.5; 640 x
+// 480, 9 x 9, k = 16: 102.1, 98.4; 481 x 321, 7 x 7, k = 98 (a longer list): 37.5, 38.3.
 __device__ __forceinline__ double canon_v(const float* __restrict__ img, int H, int W,
                                           const float* __restrict__ mask, int p, int y, int x,
                                           int t) {
@@ -242,10 +245,11 @@ __device__ __forceinline__ double canon_v(const float* __restrict__ img, int H, 
 }
 
 template <int P>
-__device__ void codes_guard_canonical(const float* __restrict__ img, int H, int W,
-                                      const float* __restrict__ omega, int k,
-                                      const float* __restrict__ mask, double tau, int2 g,
-                                      uint32_t* __restrict__ bitmask, double* sb) {
+__device__ __noinline__ void codes_guard_canonical(const float* __restrict__ img, int H, int W,
+                                                   const float* __restrict__ omega, int k,
+                                                   const float* __restrict__ mask, double tau,
+                                                   int2 g, uint32_t* __restrict__ bitmask,
+                                                   double* sb) {
     constexpr int N = P * P;
     constexpr int NL = (N + 31) / 32;  // elements per lane
     const int Wk = (k + 31) >> 5, lane = threadIdx.x & 31;
@@ -338,22 +342,15 @@ __device__ void codes_guard_canonical(const float* __restrict__ img, int H, int 
     __syncwarp();
 }
 
-template <int P>
-__global__ void __launch_bounds__(128) codes_guard_kernel(
+// The entries of the list, LE lanes each.
+template <int P, int LE>
+__device__ __forceinline__ void codes_guard_entries(
     const float* __restrict__ img, int H, int W, const float* __restrict__ omega, int k,
     const float* __restrict__ mask, const float* __restrict__ rownorm, double tau,
-    const int2* __restrict__ guard, int guard_cap, const int* __restrict__ guard_count,
-    uint32_t* __restrict__ bitmask, int* __restrict__ d_err) {
+    const int2* __restrict__ guard, int cnt, uint32_t* __restrict__ bitmask, double* sb) {
     constexpr int N = P * P;
-    constexpr int LE = 8, EW = 32 / LE;      // lanes per entry, entries per warp
+    constexpr int EW = 32 / LE;              // entries per warp
     constexpr int NL = (N + LE - 1) / LE;    // elements per lane
-    __shared__ double s_buf[4][N];           // per warp: values for the canonical sums
-    int cnt = *guard_count;
-    if (cnt > guard_cap) {
-        if (blockIdx.x == 0 && threadIdx.x == 0 && atomicCAS(d_err, 0, CS_DEVERR_GUARD_FULL) == 0)
-            d_err[1] = cnt;
-        cnt = guard_cap;
-    }
     const int Wk = (k + 31) >> 5;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, le = lane % LE;
     auto esum = [](double v) {  // sum over the entry's lanes, the same value on each
@@ -400,9 +397,29 @@ __global__ void __launch_bounds__(128) codes_guard_kernel(
             const int src = __ffs(todo) - 1;
             const int2 c = make_int2(__shfl_sync(0xffffffffu, g.x, src),
                                      __shfl_sync(0xffffffffu, g.y, src));
-            codes_guard_canonical<P>(img, H, W, omega, k, mask, tau, c, bitmask, s_buf[wib]);
+            codes_guard_canonical<P>(img, H, W, omega, k, mask, tau, c, bitmask, sb);
         }
     }
+}
+
+template <int P>
+__global__ void __launch_bounds__(128) codes_guard_kernel(
+    const float* __restrict__ img, int H, int W, const float* __restrict__ omega, int k,
+    const float* __restrict__ mask, const float* __restrict__ rownorm, double tau,
+    const int2* __restrict__ guard, int guard_cap, const int* __restrict__ guard_count,
+    uint32_t* __restrict__ bitmask, int* __restrict__ d_err) {
+    __shared__ double s_buf[4][P * P];  // per warp: values for the canonical sums
+    int cnt = *guard_count;
+    if (cnt > guard_cap) {
+        if (blockIdx.x == 0 && threadIdx.x == 0 && atomicCAS(d_err, 0, CS_DEVERR_GUARD_FULL) == 0)
+            d_err[1] = cnt;
+        cnt = guard_cap;
+    }
+    double* sb = s_buf[threadIdx.x >> 5];
+    if (cnt <= (int)gridDim.x * 3 / 2)  // (four blocks per SM)
+        codes_guard_entries<P, 32>(img, H, W, omega, k, mask, rownorm, tau, guard, cnt, bitmask, sb);
+    else
+        codes_guard_entries<P, 8>(img, H, W, omega, k, mask, rownorm, tau, guard, cnt, bitmask, sb);
 }
 
 // Patch order 1 (centre the gray values, mask, centre again, normalise):
