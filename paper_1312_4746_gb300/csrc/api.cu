@@ -228,12 +228,12 @@ cs_status cs_segment(cs_ctx* ctx, const float* f, const float* img, int H, int W
     const int nblk = seg_blocks(P, n_labels, ctx->n_sm);
     if (nblk < 1)
         return cs_set_error(ctx, CS_ERR_CUDA, "%s: the solver kernel cannot be resident", fn);
-    cs_status s = cs_ensure_scratch(ctx, seg_scratch_bytes(H, W, n_labels, nblk, ctx->n_sm,
-                                                        (float)sp->nu != 0.f));
+    const SegPlan plan = seg_plan(H, W, n_labels, ctx->n_sm, (float)sp->nu != 0.f);
+    cs_status s = cs_ensure_scratch(ctx, seg_scratch_bytes(H, W, n_labels, nblk, plan));
     if (s) return s;
     SegArgs a{f, img, H, W, n_labels, (float)sp->lambda, (float)sp->nu, (float)sp->gamma,
               sp->iterations, u, labels, reinterpret_cast<float*>(ctx->scratch), nblk,
-              ctx->d_err, ctx->n_sm};
+              ctx->d_err, plan};
     a.wait_ns = ctx->wait_ns;
     a.stall = ctx->stall == CS_STALL_SEGMENT;
     if (a.stall) ctx->stall = CS_STALL_NONE;  // one-shot

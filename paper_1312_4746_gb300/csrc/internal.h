@@ -203,6 +203,17 @@ struct SmoothArgs {
 };
 cudaError_t launch_smooth(const SmoothArgs& a, cudaStream_t st);
 
+// The solver's on-chip form for an image (kernel == nullptr: its state does not fit the
+// chip). The search over tilings takes microseconds: once per call.
+struct SegTile;
+using SegTileKernel = void (*)(SegTile);
+struct SegPlan {
+    SegTileKernel kernel = nullptr;
+    size_t smem = 0;
+    int tw = 0, th = 0, gx = 0, gy = 0, threads = 0;
+};
+SegPlan seg_plan(int H, int W, int n, int n_sm, bool sums);  // sums: nu > 0
+
 // Convex multilabel segmentation (Sec. 4) on a data term.
 struct SegArgs {
     const float* f;    // data term, n_labels x H x W
@@ -215,12 +226,12 @@ struct SegArgs {
     float* scratch;    // seg_scratch_bytes()
     int nblk;          // blocks of the cooperative launch (seg_blocks)
     int* d_err;        // device error word (timeout of a grid barrier)
-    int n_sm;
+    SegPlan plan;
     unsigned long long wait_ns = 0;  // limit of each grid-barrier wait (0: 1 s)
     bool stall = false;  // timeout-path test: the last block skips its first arrival of
                          // the iterations
 };
-size_t seg_scratch_bytes(int H, int W, int n, int nblk, int n_sm, bool sums);
+size_t seg_scratch_bytes(int H, int W, int n, int nblk, const SegPlan& plan);
 int seg_blocks(long long P, int n_labels, int n_sm);  // 0 if the kernel cannot be resident
 cudaError_t launch_segment(const SegArgs& a, cudaStream_t st);
 

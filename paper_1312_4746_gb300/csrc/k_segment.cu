@@ -305,10 +305,6 @@ int seg_grid(long long P, int n, int n_sm) {
     return k * n_sm;
 }
 
-SegPlan seg_plan(int H, int W, int n, int n_sm, bool sums) {
-    return sums ? seg_plan_mdl(H, W, n, n_sm) : seg_plan_plain(H, W, n, n_sm);
-}
-
 // Words of the exchange buffers (both parities): border ub, sums of mu, then the
 // abort flag and a word that nothing sets.
 size_t seg_exchange_words(const SegPlan& p, int n) {
@@ -319,11 +315,13 @@ size_t seg_exchange_words(const SegPlan& p, int n) {
 
 SegPlan seg_plan_plain(int H, int W, int n, int n_sm) { return seg_plan_t<false>(H, W, n, n_sm); }
 
-size_t seg_scratch_bytes(int H, int W, int n, int nblk, int n_sm, bool sums) {
-    const long long P = (long long)H * W;
-    const SegPlan pl = seg_plan(H, W, n, n_sm, sums);
-    if (pl.kernel) return 8 * seg_exchange_words(pl, n);
+SegPlan seg_plan(int H, int W, int n, int n_sm, bool sums) {
+    return sums ? seg_plan_mdl(H, W, n, n_sm) : seg_plan_plain(H, W, n, n_sm);
+}
 
+size_t seg_scratch_bytes(int H, int W, int n, int nblk, const SegPlan& plan) {
+    const long long P = (long long)H * W;
+    if (plan.kernel) return 8 * seg_exchange_words(plan, n);
     return sizeof(float) * ((size_t)4 * n * P + (size_t)P + (size_t)n * nblk) + 1024;
 }
 
@@ -337,7 +335,7 @@ cudaError_t launch_segment(const SegArgs& a, cudaStream_t st) {
     const long long P = (long long)a.H * a.W;
     const int n = a.n_labels;
     if (a.nblk < 1) return cudaErrorInvalidConfiguration;
-    const SegPlan pl = seg_plan(a.H, a.W, n, a.n_sm, a.nu != 0.f);
+    const SegPlan& pl = a.plan;
     if (pl.kernel) {
         const int G = pl.gx * pl.gy;
         const size_t per = (size_t)G * n * seg_border(pl.tw, pl.th);

@@ -26,14 +26,6 @@ struct SegTile {
     bool stall;
 };
 
-using SegTileKernel = void (*)(SegTile);
-
-struct SegPlan {
-    SegTileKernel kernel = nullptr;
-    size_t smem = 0;
-    int tw = 0, th = 0, gx = 0, gy = 0, threads = 0;
-};
-
 // the tilings (kernel == nullptr: the state does not fit the chip)
 SegPlan seg_plan_plain(int H, int W, int n, int n_sm);  // nu = 0
 SegPlan seg_plan_mdl(int H, int W, int n, int n_sm);    // nu > 0
