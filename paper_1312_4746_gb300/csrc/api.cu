@@ -565,6 +565,7 @@ void cs_lik_plan(LikPlan& L, int H, int W, int k, int n_labels,
     L.tc_form = prm->precision != CS_FP32;
     L.tex8 = prm->precision == CS_FP8;
     L.persample = prm->mode == CS_MODE_PERSAMPLE;
+    L.few = !L.tc_form && plain_few(H, W, k, n_labels, label_off, L.persample);
     for (int i = 0; i <= n_labels; ++i) L.offs.v[i] = label_off[i];
     L.offs.v[n_labels + 1] = 0;
     for (int i = 0; i < n_labels; ++i)
@@ -575,7 +576,7 @@ void cs_lik_plan(LikPlan& L, int H, int W, int k, int n_labels,
     L.n_chunks = 0;
     for (int i = 0; i < n_labels; ++i) L.n_chunks += (label_off[i + 1] - label_off[i] + 4095) / 4096;
     L.stage_bytes = L.tc_form ? tc_copy_bytes(k, L.tex8, L.persample)
-                              : plain_tile_bytes(k, L.persample);
+                              : plain_tile_bytes(k, L.persample, L.few);
 }
 
 void cs_lik_carve(Carve& c, LikPlan& L, int32_t* dist2) {
@@ -652,6 +653,7 @@ SumArgs cs_sum_args(cs_ctx* ctx, const LikPlan& L, const float* img, const uint3
     a.rho_var = prm->rho_variance != 0;
     a.neglog = neglog;
     a.post = post;
+    a.few = L.few;
     a.d_err = ctx->d_err;
     a.wait_ns = ctx->wait_ns;
     return a;
@@ -725,7 +727,7 @@ static cudaError_t enqueue_sum(cs_ctx* ctx, const LikPlan& L, const float* img,
         StageTimer tm(ctx, CS_STAGE_GATHER, st);
         e = L.tc_form ? launch_sum_tc_prepare(T, sorted, st)
                       : launch_plain_tiles(img, L.H, L.W, bitmask, L.k, L.n_labels, L.d_off,
-                                           sample_pix, L.total_tiles, L.persample, L.t.blob, st);
+                                           sample_pix, L.total_tiles, L.persample, L.few, L.t.blob, st);
         // (the smooth texture has representatives of its own)
         if (e == cudaSuccess && prm->mode == CS_MODE_FACTORISED)
             e = launch_majority(L.H, L.W, bitmask, L.k, L.n_labels, L.d_off, sample_pix, L.t.rep, st);
@@ -735,7 +737,7 @@ static cudaError_t enqueue_sum(cs_ctx* ctx, const LikPlan& L, const float* img,
     StageTimer tm(ctx, CS_STAGE_SUM, st);
     if (L.tc_form) return launch_sum_tc_run(T, st);
     SumArgs a = cs_sum_args(ctx, L, img, bitmask, prm, neglog, post);
-    a.stall = L.persample && ctx->stall == CS_STALL_PLAIN;
+    a.stall = L.persample && !L.few && ctx->stall == CS_STALL_PLAIN;
     if (a.stall) ctx->stall = CS_STALL_NONE;
     return launch_sum_plain(a, st);
 }
@@ -829,7 +831,7 @@ cudaError_t cs_enqueue_prepare(cs_ctx* ctx, const LikPlan& L, const float* img,
         e = launch_majority(L.H, L.W, bitmask, L.k, L.n_labels, L.d_off, sample_pix, L.t.rep, st);
     if (e != cudaSuccess || L.tc_form) return e;
     return launch_plain_tiles(img, L.H, L.W, bitmask, L.k, L.n_labels, L.d_off, sample_pix,
-                              L.total_tiles, L.persample, L.t.blob, st);
+                              L.total_tiles, L.persample, L.few, L.t.blob, st);
 }
 
 // exact plain sum over a device pixel list (after cs_enqueue_prepare): with

@@ -177,7 +177,7 @@ static cudaError_t enqueue_run(cs_batch* b, cudaStream_t st) {
             e = launch_tc_prepare(T, ss);
         } else {
             e = launch_plain_tiles(m.d.img, L.H, L.W, m.codes.bitmask, L.k, L.n_labels, L.d_off,
-                                   m.d.sample_pix, L.total_tiles, L.persample, L.t.blob, ss);
+                                   m.d.sample_pix, L.total_tiles, L.persample, L.few, L.t.blob, ss);
             if (e == cudaSuccess)
                 e = launch_sum_plain(cs_sum_args(ctx, L, m.d.img, m.codes.bitmask, &b->prm,
                                                  m.d.neglog, m.d.post), ss);

@@ -330,6 +330,7 @@ struct SumArgs {
     const int* list_count = nullptr;
     int list_cap = 0;
     float* T_out = nullptr;
+    bool few = false;      // plain_few
     int* d_err = nullptr;  // device error word (a wait for the tensor cores that gave up)
     unsigned long long wait_ns = 0;  // limit of each wait for the tensor cores (0: 1 s)
     bool stall = false;  // timeout-path test: the last block waits for what nothing completes
@@ -338,11 +339,13 @@ struct SumArgs {
 // the label offsets at d_label_off + n_labels + 1)
 cudaError_t launch_sum_plain(const SumArgs& a, cudaStream_t st);
 int plain_tiles_per_label(int m);
-size_t plain_tile_bytes(int k, bool persample);
+// the few-samples form of the plain sum (k_sum.cu): chosen by the plan
+bool plain_few(int H, int W, int k, int n_labels, const int32_t* label_off, bool persample);
+size_t plain_tile_bytes(int k, bool persample, bool few);
 cudaError_t launch_plain_tiles(const float* img, int H, int W, const uint32_t* bitmask, int k,
                                int n_labels, const int32_t* d_label_off,
                                const int32_t* sample_pix, int total_tiles, bool persample,
-                               uint8_t* blob, cudaStream_t st);
+                               bool few, uint8_t* blob, cudaStream_t st);
 
 struct TcImage;
 
@@ -350,6 +353,7 @@ struct TcImage;
 struct LikPlan {
     int H, W, k, n_labels, S, total_tiles, n_chunks;
     bool tc_form, tex8, persample;
+    bool few;  // plain form: plain_few
     size_t stage_bytes;
     OffsetsParam offs;  // label offsets then first sample tile of each label
     int32_t* d_off;

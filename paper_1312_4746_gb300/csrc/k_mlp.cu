@@ -651,9 +651,10 @@ __device__ void eval_pixel(const FwdArgs& a, long long q, float (&z)[64], const 
     const float log_col_norm = 1.5f * logf(6.283185307179586f * a.sigma_c2);
     uint32_t bx[8];
     for (int w = 0; w < 8; ++w)
-        bx[w] = (a.mode == CS_MODE_FACTORISED && w < a.Wk)
-                    ? a.bitmask[q * a.Wk + w] & code_mask(w, a.k)
-                    : 0u;
+        bx[w] = (a.mode == CS_MODE_FACTORISED && w < a.Wk) ? a.bitmask[q * a.Wk + w] : 0u;
+    const int pad = a.mode == CS_MODE_FACTORISED  // bits that are no codes
+                        ? __popc(a.bitmask[q * a.Wk + a.Wk - 1] & ~code_mask(a.Wk - 1, a.k))
+                        : 0;
     float tmax = -INFINITY;
     float tex[64];  // factorised mode: the texture exponents -h_j / beta_j
     for (int j = 0; j < n; ++j) {
@@ -662,7 +663,7 @@ __device__ void eval_pixel(const FwdArgs& a, long long q, float (&z)[64], const 
         z[j] = T - logf((float)(a.label_off[j + 1] - a.label_off[j])) -
                logf(6.283185307179586f * (a.rho_var ? rho : rho * rho)) - log_col_norm;
         if (a.mode == CS_MODE_FACTORISED) {
-            int h = 0;
+            int h = -pad;
             for (int w = 0; w < a.Wk; ++w) h += __popc(bx[w & 7] ^ a.rep[j * a.Wk + w]);
             tex[j] = -(float)h / (a.kappa_beta * rho);
             tmax = fmaxf(tmax, tex[j]);

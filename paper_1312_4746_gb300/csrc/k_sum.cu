@@ -32,6 +32,11 @@
 // 32 samples. It keeps an online log-sum-exp per pixel: a running maximum per 16
 // samples and a TwoSum-compensated running sum per 32; the two threads of a
 // pixel merge at the label's end. A second kernel normalises over the labels.
+//
+// Few samples per label on enough pixels (plain_few) take sum_few_kernel instead: a
+// thread per pixel over all labels, the TSM by population counts, the normalisation at
+// its end. There the operand rows, the waits and the merge of every (pixels, label)
+// unit and the tiles' padding cost more than the population counts.
 #include <cstdint>
 #include <type_traits>
 
@@ -133,12 +138,15 @@ __device__ __forceinline__ uint32_t e4m3_minus(int v) {
     return 0x80u | (uint32_t)(ex + 7) << 3 | (uint32_t)(((v << 3) >> ex) & 7);
 }
 
+// Bytes of a tile of the few-samples form: the planes, then the codes' words as planes.
+__host__ __device__ constexpr int few_tile_bytes(int Wk) { return (5 + Wk) * TS * 4; }
+
 // Sample tiles: one thread per (tile, sample). Padded samples lie far away (their
-// terms vanish) and have no codes.
+// terms vanish) and have no codes. words > 0: the few-samples form's layout.
 __global__ void __launch_bounds__(256) plain_tiles_kernel(
     const float* __restrict__ img, int W, long long P, const uint32_t* __restrict__ bitmask, int Wk,
     const int32_t* __restrict__ label_off, const int32_t* __restrict__ tile_off, int n_labels,
-    const int32_t* __restrict__ sample_pix, int total_tiles, int k, int KS,
+    const int32_t* __restrict__ sample_pix, int total_tiles, int k, int KS, int words,
     uint8_t* __restrict__ blob) {
     const long long gid = blockIdx.x * 256ll + threadIdx.x;
     if (gid >= (long long)total_tiles * TS) return;
@@ -150,7 +158,7 @@ __global__ void __launch_bounds__(256) plain_tiles_kernel(
     }
     const int s = label_off[lo] + (tile - tile_off[lo]) * TS + r;
     const bool ok = s < label_off[lo + 1];
-    uint8_t* base = blob + (size_t)tile * tile_bytes(KS);
+    uint8_t* base = blob + (size_t)tile * (words ? few_tile_bytes(words) : tile_bytes(KS));
     float* f = reinterpret_cast<float*>(base);
     int pix = ok ? sample_pix[s] : 0;
     if (pix < 0 || pix >= P) pix = 0;  // reported by the distance transform's seed pass
@@ -158,6 +166,9 @@ __global__ void __launch_bounds__(256) plain_tiles_kernel(
     f[TS + r] = ok ? (float)(pix / W) : 0.f;
 #pragma unroll
     for (int c = 0; c < 3; ++c) f[(2 + c) * TS + r] = ok ? img[(size_t)pix * 3 + c] : 0.f;
+    for (int w = 0; w < words; ++w)
+        reinterpret_cast<uint32_t*>(f)[(5 + w) * TS + r] =
+            ok ? bitmask[(size_t)pix * Wk + w] & code_mask(w, k) : 0u;
     for (int w = 0; w < KS; ++w) {
         uint32_t bits = ok && w < Wk ? bitmask[(size_t)pix * Wk + w] & code_mask(w, k) : 0u;
         for (int c = k; c < k + 2; ++c)  // the columns of -|b_x|
@@ -470,40 +481,148 @@ __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
     }
 }
 
-// Label normalisation (and the factorised texture posterior), one thread per item.
+// Label normalisation (and the factorised texture posterior) of pixel q.
+__device__ __forceinline__ void normalise_plain(const SumArgs& a, long long P, long long q) {
+    if (a.mode == CS_MODE_FACTORISED) {
+        const uint32_t* bx = a.bitmask + (size_t)q * a.Wk;
+        const int pad = __popc(bx[a.Wk - 1] & ~code_mask(a.Wk - 1, a.k));  // bits that are no codes
+        auto logit = [&](int i) {
+            float rho, nA, nB;
+            label_consts(a.dist2[(size_t)i * P + q], a.alpha, a.d_min, a.kappa_beta, a.rho_var,
+                         rho, nA, nB);
+            int h = -pad;
+            for (int w = 0; w < a.Wk; ++w) h += __popc(bx[w] ^ a.t.rep[i * a.Wk + w]);
+            return nB * (float)h;
+        };
+        float tmax = -INFINITY;
+        for (int i = 0; i < a.n_labels; ++i) tmax = fmaxf(tmax, logit(i));
+        float ts = 0.f;
+        for (int i = 0; i < a.n_labels; ++i) ts += ex2(logit(i) - tmax);
+        const float tlse2 = tmax + log2f(ts);
+        for (int i = 0; i < a.n_labels; ++i)  // texture log-posterior, natural log
+            a.neglog[(size_t)i * P + q] -= (logit(i) - tlse2) * LN2;
+    }
+    if (!a.post) return;
+    float lmax = -INFINITY;
+    for (int i = 0; i < a.n_labels; ++i) lmax = fmaxf(lmax, -a.neglog[(size_t)i * P + q]);
+    float ls = 0.f;
+    for (int i = 0; i < a.n_labels; ++i) ls += expf(-a.neglog[(size_t)i * P + q] - lmax);
+    const float lse = lmax + logf(ls);
+    for (int i = 0; i < a.n_labels; ++i)
+        a.post[(size_t)i * P + q] = expf(-a.neglog[(size_t)i * P + q] - lse);
+}
 __global__ void __launch_bounds__(256) normalise_plain_kernel(SumArgs a) {
     const long long P = (long long)a.H * a.W;
     const long long n_items = a.pix_list ? (long long)min(*a.list_count, a.list_cap) : P;
     for (long long it = blockIdx.x * 256ll + threadIdx.x; it < n_items;
-         it += (long long)gridDim.x * 256) {
-        const long long q = a.pix_list ? (long long)a.pix_list[it] : it;
-        if (a.mode == CS_MODE_FACTORISED) {
-            const uint32_t* bx = a.bitmask + (size_t)q * a.Wk;
-            const int pad = __popc(bx[a.Wk - 1] & ~code_mask(a.Wk - 1, a.k));  // bits that are no codes
-            auto logit = [&](int i) {
-                float rho, nA, nB;
-                label_consts(a.dist2[(size_t)i * P + q], a.alpha, a.d_min, a.kappa_beta, a.rho_var,
-                             rho, nA, nB);
-                int h = -pad;
-                for (int w = 0; w < a.Wk; ++w) h += __popc(bx[w] ^ a.t.rep[i * a.Wk + w]);
-                return nB * (float)h;
-            };
-            float tmax = -INFINITY;
-            for (int i = 0; i < a.n_labels; ++i) tmax = fmaxf(tmax, logit(i));
-            float ts = 0.f;
-            for (int i = 0; i < a.n_labels; ++i) ts += ex2(logit(i) - tmax);
-            const float tlse2 = tmax + log2f(ts);
-            for (int i = 0; i < a.n_labels; ++i)  // texture log-posterior, natural log
-                a.neglog[(size_t)i * P + q] -= (logit(i) - tlse2) * LN2;
+         it += (long long)gridDim.x * 256)
+        normalise_plain(a, P, a.pix_list ? (long long)a.pix_list[it] : it);
+}
+
+// The few-samples form: a thread per pixel, all labels in turn; sums as in the general
+// form's comment, with the running maximum and the TwoSum per 16 samples. Bound: with
+// the texture, the population counts (WK a pair, 16 per clock and SM). WK: words of the
+// texture (0: none in the pairs). Measured, sum and normalisation, us, against the
+// general form: 2048 x 1024, 4 labels of 10 samples, k = 50: 190, 865; factorised: 232,
+// 607; 481 x 321, 5 x 60, k = 98: 66, 99; 320 x 240, 64 x 40, k = 98: 318, 560.
+constexpr int FEW_THREADS = 128;
+template <int WK>
+__global__ void __launch_bounds__(FEW_THREADS) sum_few_kernel(SumArgs a) {
+    constexpr int TB = few_tile_bytes(WK), CH = 16;
+    __shared__ __align__(16) float s_tile[TB / 4];  // x, y, r, g, b, words
+    const uint32_t* s_bits = reinterpret_cast<const uint32_t*>(s_tile + 5 * TS);
+    const long long P = (long long)a.H * a.W;
+    const int tid = threadIdx.x;
+    const float nC = -LOG2E / (2.f * a.sigma_c2);
+    const float log_col_norm = 1.5f * logf(6.283185307179586f * a.sigma_c2);
+    const int n_items = a.pix_list ? min(*a.list_count, a.list_cap) : (int)P;
+    const int32_t* tile_off = a.d_label_off + a.n_labels + 1;
+    // a tile is read ahead into registers while the one before is summed (the labels'
+    // tiles follow one another)
+    constexpr int NV = (TB / 16 + FEW_THREADS - 1) / FEW_THREADS;
+    const int n_tiles = tile_off[a.n_labels];
+    uint4 ahead[NV];
+    auto read = [&](int T) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int c = tid + v * FEW_THREADS;
+            if (c < TB / 16 && T < n_tiles)
+                ahead[v] = reinterpret_cast<const uint4*>(a.t.blob + (size_t)T * TB)[c];
         }
-        if (!a.post) continue;
-        float lmax = -INFINITY;
-        for (int i = 0; i < a.n_labels; ++i) lmax = fmaxf(lmax, -a.neglog[(size_t)i * P + q]);
-        float ls = 0.f;
-        for (int i = 0; i < a.n_labels; ++i) ls += expf(-a.neglog[(size_t)i * P + q] - lmax);
-        const float lse = lmax + logf(ls);
-        for (int i = 0; i < a.n_labels; ++i)
-            a.post[(size_t)i * P + q] = expf(-a.neglog[(size_t)i * P + q] - lse);
+    };
+    for (long long base = (long long)blockIdx.x * FEW_THREADS; base < n_items;
+         base += (long long)gridDim.x * FEW_THREADS) {
+        read(0);
+        const int it = (int)base + tid;
+        const bool live = it < n_items;
+        const int q = live ? (a.pix_list ? a.pix_list[it] : it) : 0;
+        const float px = (float)(q % a.W), py = (float)(q / a.W);
+        const float* I = a.img + (size_t)q * 3;
+        const float pr = I[0], pg = I[1], pb = I[2];
+        uint32_t bits[WK > 0 ? WK : 1];
+#pragma unroll
+        for (int w = 0; w < WK; ++w) bits[w] = a.bitmask[(size_t)q * WK + w] & code_mask(w, a.k);
+        for (int i = 0; i < a.n_labels; ++i) {
+            float rho, nA, nB, M = LOWEST, S = 0.f, Cc = 0.f;
+            label_consts(a.dist2[(size_t)i * P + q], a.alpha, a.d_min, a.kappa_beta, a.rho_var, rho,
+                         nA, nB);
+            const int m = a.d_label_off[i + 1] - a.d_label_off[i];
+            for (int T = tile_off[i]; T < tile_off[i + 1]; ++T) {
+                __syncthreads();
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    const int c = tid + v * FEW_THREADS;
+                    if (c < TB / 16) reinterpret_cast<uint4*>(s_tile)[c] = ahead[v];
+                }
+                __syncthreads();
+                read(T + 1);
+                const int nvalid = min(TS, m - (T - tile_off[i]) * TS);
+                for (int c0 = 0; c0 < nvalid; c0 += CH) {
+                    float e[CH], mx = LOWEST;
+#pragma unroll
+                    for (int c = 0; c < CH; ++c) {
+                        const int j = c0 + c;
+                        const float dx = px - s_tile[j], dy = py - s_tile[TS + j];
+                        const float dr = pr - s_tile[2 * TS + j], dg = pg - s_tile[3 * TS + j],
+                                    db = pb - s_tile[4 * TS + j];
+                        const float d2 = fmaf(dx, dx, dy * dy);
+                        const float c2 = fmaf(dr, dr, fmaf(dg, dg, db * db));
+                        float col = nC * c2;
+                        if (WK > 0) {
+                            int h = 0;
+#pragma unroll
+                            for (int w = 0; w < WK; ++w) h += __popc(bits[w] ^ s_bits[w * TS + j]);
+                            col = fmaf(nC, c2, nB * (float)h);
+                        }
+                        e[c] = fmaf(nA, d2, col);
+                        mx = fmaxf(mx, e[c]);
+                    }
+                    if (mx > M) {
+                        const float sc = ex2(M - mx);
+                        S *= sc;
+                        Cc *= sc;
+                        M = mx;
+                    }
+                    float ts = 0.f;
+#pragma unroll
+                    for (int c = 0; c < CH; ++c) ts += ex2(e[c] - M);
+                    // TwoSum: S + ts = s + err exactly
+                    const float s = S + ts, bb = s - S;
+                    Cc += (S - (s - bb)) + (ts - bb);
+                    S = s;
+                }
+            }
+            if (!live) continue;
+            const float lse = (M + log2f(S + Cc)) * LN2;
+            if (a.T_out) {  // log kernel sum only (surrogate targets), compact layout
+                a.T_out[(size_t)i * a.list_cap + it] = lse;
+                continue;
+            }
+            const float s2 = a.rho_var ? rho : rho * rho;
+            a.neglog[(size_t)i * P + q] =
+                -(lse - logf((float)m) - logf(6.283185307179586f * s2) - log_col_norm);
+        }
+        if (live && !a.T_out) normalise_plain(a, P, q);
     }
 }
 
@@ -530,23 +649,50 @@ cudaError_t with_steps(int KS, F&& f) {
 
 int plain_tiles_per_label(int m) { return (m + TS - 1) / TS; }
 
-size_t plain_tile_bytes(int k, bool persample) {
-    return (size_t)tile_bytes(persample ? steps_for(k) : 0);
+// The few-samples form? Its cost goes with the samples, padded to 16 per label, and
+// their words; the general form's with 64-sample tiles and units. With the texture the
+// two meet near 200 samples a label at four words, 128 at six; and the few-samples form
+// needs pixels, which is all it works on in parallel. Measured, tiles, sum and
+// normalisation, us, few and general (k = 98; samples per label x labels):
+//   481 x 321: 16 x 5 36, 105; 64 x 5 71, 105; 130 x 5 138, 161; 200 x 5 191, 191
+//   320 x 240: 130 x 16 .90 of the general form's; 240 x 180: 64 x 16 .91, 100 x 16
+//   1.17; 200 x 100: 16 x 16 .69, 40 x 16 1.06; 96 x 64: 64 x 2 .88, 100 x 2 1.07
+//   (factorised, 481 x 321: 16 x 5 .51, 64 x 5 .77, 200 x 5 .85)
+bool plain_few(int H, int W, int k, int n_labels, const int32_t* label_off, bool persample) {
+    const long long P = (long long)H * W;
+    long long padded = 0;
+    for (int i = 0; i < n_labels; ++i) padded += (label_off[i + 1] - label_off[i] + 15) / 16 * 16;
+    const int most = persample && (k + 31) / 32 > 4 ? 768 / ((k + 31) / 32) : 192;
+    return padded <= (long long)most * n_labels && (P >= 60000 || 40 * padded <= P);
+}
+
+size_t plain_tile_bytes(int k, bool persample, bool few) {
+    return few ? (size_t)few_tile_bytes(persample ? (k + 31) / 32 : 0)
+               : (size_t)tile_bytes(persample ? steps_for(k) : 0);
 }
 
 cudaError_t launch_plain_tiles(const float* img, int H, int W, const uint32_t* bitmask, int k,
                                int n_labels, const int32_t* d_label_off,
                                const int32_t* sample_pix, int total_tiles, bool persample,
-                               uint8_t* blob, cudaStream_t st) {
+                               bool few, uint8_t* blob, cudaStream_t st) {
     const long long n = (long long)total_tiles * TS;
     plain_tiles_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
         img, W, (long long)H * W, bitmask, (k + 31) / 32, d_label_off, d_label_off + n_labels + 1,
-        n_labels, sample_pix, total_tiles, k, persample ? steps_for(k) : 0, blob);
+        n_labels, sample_pix, total_tiles, k, persample && !few ? steps_for(k) : 0,
+        persample && few ? (k + 31) / 32 : 0, blob);
     return cudaGetLastError();
 }
 
 cudaError_t launch_sum_plain(const SumArgs& a, cudaStream_t st) {
     const long long n = a.pix_list ? (long long)a.list_cap : (long long)a.H * a.W;
+    if (a.few)
+        return with_steps(a.mode == CS_MODE_PERSAMPLE ? a.Wk : 0, [&](auto wk) {
+            constexpr int WK = decltype(wk)::value;
+            long long blocks = (n + FEW_THREADS - 1) / FEW_THREADS;
+            if (a.pix_list && blocks > 152 * 16) blocks = 152 * 16;  // grid-stride over the list
+            sum_few_kernel<WK><<<(unsigned)(blocks < 1 ? 1 : blocks), FEW_THREADS, 0, st>>>(a);
+            return cudaGetLastError();
+        });
     const cudaError_t e = with_steps(steps_of(a), [&](auto ks) {
         constexpr int KS = decltype(ks)::value;
         auto run = [&](auto pt) {

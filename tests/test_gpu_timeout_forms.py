@@ -60,10 +60,11 @@ def test_segment_forms(env, n, nu):
     assert torch.equal(out["u"], ref["u"]) and torch.equal(out["labels"], ref["labels"])
 
 
-@pytest.mark.parametrize("H,W", [(64, 96), (152, 257)])  # one and two operand tiles per block
-def test_plain_sum(env, H, W):
+@pytest.mark.parametrize("H,W,m", [(64, 96, [70, 5, 64, 130]),  # one operand tile per block
+                                   (152, 257, [400, 5, 64, 430])])  # two
+def test_plain_sum(env, H, W, m):
     cs, ctx, torch = env
-    pr = synth.make_problem(H, W, 4, [70, 5, 64, 130], p=5, k=50, seed=77)
+    pr = synth.make_problem(H, W, 4, m, p=5, k=50, seed=77)
     img, om, mask, smp = (torch.from_numpy(np.ascontiguousarray(a)).to("cuda:0")
                           for a in (pr.image, pr.omega, pr.mask, pr.sample_pix))
     prm = cs.Params.from_synth(pr.params)
