@@ -592,20 +592,20 @@ __device__ __forceinline__ void ct_set_error(int* d_err, int site) {
 }
 
 // The 16 codes of chunk c to the callers' arrays: `codes` (k per pixel), and the
-// first chunk to `lead16` (zero beyond k, also where a patch holds a NaN or infinity,
-// whose products with the operator's zero padding rows are NaN).
+// first chunk to `lead16` (beyond k zero, or NaN from a patch that is not finite, whose
+// products with the operator's zero padding rows are NaN: see zero_lead16).
 __device__ __forceinline__ void store_codes(const uint32_t (&v)[16], int c, bool live, int pix, int k,
                                             float* __restrict__ codes, float* __restrict__ lead16) {
     if (lead16 && c == 0 && live) {
         float4* d = reinterpret_cast<float4*>(lead16 + (size_t)pix * 16);
-        auto code = [&](int e) { return e < k ? __uint_as_float(v[e]) : 0.f; };
         if ((reinterpret_cast<uintptr_t>(d) & 15) == 0) {
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                d[q] = make_float4(code(4 * q), code(4 * q + 1), code(4 * q + 2), code(4 * q + 3));
+                d[q] = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
+                                   __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
         } else {
 #pragma unroll
-            for (int e = 0; e < 16; ++e) lead16[(size_t)pix * 16 + e] = code(e);
+            for (int e = 0; e < 16; ++e) lead16[(size_t)pix * 16 + e] = __uint_as_float(v[e]);
         }
     }
     if (codes && live) {
@@ -613,6 +613,13 @@ __device__ __forceinline__ void store_codes(const uint32_t (&v)[16], int c, bool
         for (int e = 0; e < 16; ++e)
             if (16 * c + e < k) codes[(size_t)pix * k + 16 * c + e] = __uint_as_float(v[e]);
     }
+}
+
+// The pixel's places of lead16 beyond k, after store_codes of chunk 0 (by the same
+// thread; out of its loop, whose code a selection per code slows by 8% at k = 200).
+__device__ __forceinline__ void zero_lead16(bool live, int pix, int k, float* __restrict__ lead16) {
+    if (lead16 && live)
+        for (int j = k; j < 16; ++j) lead16[(size_t)pix * 16 + j] = 0.f;
 }
 
 template <int P>
@@ -805,6 +812,7 @@ __global__ void __launch_bounds__(128, 4) codes_tc_kernel(
             }
         }
         if (live && whole) guard_push(guard, guard_cap, guard_count, pix, -1);
+        zero_lead16(live, pix, k, lead16);
     } else if (tid == 0 && *s_flag) {
         // MMAs still in flight: they must finish before the tensor memory is freed
         tc::mbar_wait(bars + 1, 0, tc::globaltimer() + wait_ns);
@@ -855,10 +863,14 @@ __host__ __device__ constexpr CpOff cp_off(int np) {
 // another role has aborted.
 __device__ __forceinline__ bool cp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                         int* d_err, int site, uint64_t wait_ns) {
-    const uint64_t deadline = tc::globaltimer() + wait_ns;
+    uint64_t deadline = 0;
     for (uint32_t n = 0;; ++n) {
         if (tc::mbar_try_wait(bar, parity, 1000u)) return true;
-        if ((n & 63u) == 63u && (*abort_flag || tc::globaltimer() > deadline)) break;
+        if ((n & 63u) == 63u) {
+            const uint64_t now = tc::globaltimer();
+            if (deadline == 0) deadline = now + wait_ns;
+            if (*abort_flag || now > deadline) break;
+        }
     }
     *abort_flag = 1;
     ct_set_error(d_err, site);
@@ -873,7 +885,11 @@ __device__ __forceinline__ bool cp_wait_warp(uint64_t* bar, uint32_t parity,
     return __all_sync(0xffffffffu, cp_wait(bar, parity, abort_flag, d_err, site, wait_ns));
 }
 
-template <int P>
+// OUT: 0 neither `codes` nor `lead16` is wanted (the epilogue is thresholds only), 1
+// `lead16`, 2 `codes` (and perhaps `lead16`). Tests of the pointers in the epilogue's
+// loop cost 8 to 12% where its 16-code chunks are many (1023 x 769, 3 x 3, k = 200: 160
+// us with them, 140 without).
+template <int P, int OUT>
 __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kernel(
     const float* __restrict__ img, int H, int W, const uint8_t* __restrict__ blob, int k, int np,
     const float* __restrict__ mask, const float* __restrict__ rownorm, float tau_f,
@@ -1070,7 +1086,8 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
                         tc::tmem_ld16(lrow + (uint32_t)(b * ncols) + 16u * c, v);
                         tc::tmem_ld_wait();
                         threshold16(v, 16 * h, s_rn + 16 * c, ebase, tau_f, tau_slack, word, gword);
-                        store_codes(v, c, live, pix, k, codes, lead16);
+                        if (OUT)
+                            store_codes(v, c, live, pix, k, OUT == 2 ? codes : nullptr, lead16);
                     }
                 }
                 const uint32_t m = code_mask(wd, k);
@@ -1081,6 +1098,7 @@ __global__ void __launch_bounds__(cp_threads(P), P <= 7 ? 2 : 1) codes_tcp_kerne
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(t_empty + b);
             if (live && whole && eg == 0) guard_push(guard, guard_cap, guard_count, pix, -1);
+            if (OUT && eg == 0) zero_lead16(live, pix, k, lead16);
         }
     } else if (lane == 0) {
         // ---------------------------------------------------------- MMA issuer
@@ -1174,7 +1192,10 @@ cudaError_t launch_tc_p(const CodesArgs& a, cudaStream_t st) {
     }
     const size_t floor_b = 233472 / (per_sm + 1) - 1024 + 16;  // no further CTA fits
     if (psmem < floor_b) psmem = floor_b;
-    e = cs_smem_limit((const void*)codes_tcp_kernel<P>, 233472 - 1024);  // one CTA per SM takes all
+    const auto kernel = a.codes    ? codes_tcp_kernel<P, 2>
+                        : a.lead16 ? codes_tcp_kernel<P, 1>
+                                   : codes_tcp_kernel<P, 0>;
+    e = cs_smem_limit((const void*)kernel, 233472 - 1024);  // one CTA per SM takes all
     if (e != cudaSuccess) return e;
     int dev = 0, n_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1182,7 +1203,7 @@ cudaError_t launch_tc_p(const CodesArgs& a, cudaStream_t st) {
         return e;
     const int ntiles = ((a.W + CT_W - 1) / CT_W) * ((a.H + CT_H - 1) / CT_H);
     const int grid = ntiles < per_sm * n_sm ? ntiles : per_sm * n_sm;
-    codes_tcp_kernel<P><<<grid, cp_threads(P), psmem, st>>>(
+    kernel<<<grid, cp_threads(P), psmem, st>>>(
         a.img, a.H, a.W, a.omega_blob, a.k, np, a.mask, a.rownorm, tau_f, slack, a.codes,
         a.lead16, a.bitmask, a.guard, a.guard_cap, a.guard_count, a.d_err, wait_ns, a.stall);
     return cudaGetLastError();
