@@ -155,14 +155,14 @@ def pair_ops(form: str, Wk: int) -> dict:
     """Algorithmic operations per pixel x sample pair.
 
     fp32 (CUDA cores): location 2 sub + mul + fma, colour 3 sub + mul + 2 fma,
-    combine 3, running max, exponent offset and sum (16 FP32); one ex2. The
-    texture distance comes from the tensor cores.
+    combine 3, exponent offset and sum (15 FP32); one ex2. The running maximum
+    is the integer pipe's, the texture distance the tensor cores'.
     tensor-core forms: the dot products run on the tensor cores; the CUDA
     cores do 2 FFMA (texture/colour scale, location scale) and one add per
     pair (3 FP32) and one ex2.
     """
     if form == "fp32":
-        return {"fp32": 16, "mufu": 1}
+        return {"fp32": 15, "mufu": 1}
     return {"fp32": 3, "mufu": 1}
 
 

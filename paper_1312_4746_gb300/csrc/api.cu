@@ -654,6 +654,7 @@ SumArgs cs_sum_args(cs_ctx* ctx, const LikPlan& L, const float* img, const uint3
     a.neglog = neglog;
     a.post = post;
     a.few = L.few;
+    a.n_sm = ctx->n_sm;
     a.d_err = ctx->d_err;
     a.wait_ns = ctx->wait_ns;
     return a;

@@ -331,6 +331,7 @@ struct SumArgs {
     int list_cap = 0;
     float* T_out = nullptr;
     bool few = false;      // plain_few
+    int n_sm = 0;
     int* d_err = nullptr;  // device error word (a wait for the tensor cores that gave up)
     unsigned long long wait_ns = 0;  // limit of each wait for the tensor cores (0: 1 s)
     bool stall = false;  // timeout-path test: the last block waits for what nothing completes

@@ -200,10 +200,10 @@ __device__ __forceinline__ bool plain_wait(uint64_t* bars, MmaPhase p, uint64_t 
 
 // KS: 32-column steps of the texture (0: no texture in the pairs, the factorised
 // and smooth forms); PT: 128-pixel operand tiles per CTA (one where two would
-// leave SMs without a CTA). Bound: the FP32 pipe (14 packed operations per two
-// pairs: 0.58 ms at 481 x 321, 10,000 samples). Measured there: 0.99 ms, against
-// 1.65 ms with population counts, nine shared-memory words read per pair and
-// scalar arithmetic.
+// leave SMs without a CTA). Bound: the FP32 pipe (15 packed operations per two pairs
+// with the texture, the running maximum beside them in the integer pipe: 0.63 ms at
+// 481 x 321, 10,000 samples). Measured there: 0.97 ms, against 1.65 ms with population
+// counts, nine shared-memory words read per pair and scalar arithmetic.
 template <int KS, int PT>
 __global__ void __launch_bounds__(THREADS, 2) sum_plain_kernel(SumArgs a) {
     constexpr bool TEX = KS > 0;
@@ -685,11 +685,12 @@ cudaError_t launch_plain_tiles(const float* img, int H, int W, const uint32_t* b
 
 cudaError_t launch_sum_plain(const SumArgs& a, cudaStream_t st) {
     const long long n = a.pix_list ? (long long)a.list_cap : (long long)a.H * a.W;
+    const long long most = 16ll * a.n_sm;
     if (a.few)
         return with_steps(a.mode == CS_MODE_PERSAMPLE ? a.Wk : 0, [&](auto wk) {
             constexpr int WK = decltype(wk)::value;
             long long blocks = (n + FEW_THREADS - 1) / FEW_THREADS;
-            if (a.pix_list && blocks > 152 * 16) blocks = 152 * 16;  // grid-stride over the list
+            if (a.pix_list && blocks > most) blocks = most;  // grid-stride over the list
             sum_few_kernel<WK><<<(unsigned)(blocks < 1 ? 1 : blocks), FEW_THREADS, 0, st>>>(a);
             return cudaGetLastError();
         });
@@ -703,19 +704,19 @@ cudaError_t launch_sum_plain(const SumArgs& a, cudaStream_t st) {
                 sum_plain_kernel<KS, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             if (e2 != cudaSuccess) return e2;
             long long blocks = (n + 128 * PT - 1) / (128 * PT) * a.n_labels;
-            if (a.pix_list && blocks > 152 * 16) blocks = 152 * 16;  // grid-stride over the list
+            if (a.pix_list && blocks > most) blocks = most;  // grid-stride over the list
             if (blocks > 0x7fffffffll) blocks = 0x7fffffffll;
             sum_plain_kernel<KS, PT><<<(unsigned)(blocks < 1 ? 1 : blocks), THREADS, smem, st>>>(a);
             return cudaGetLastError();
         };
         // two operand tiles share the samples' reads; one where the units of two
         // would not fill the SMs twice
-        return (n + 255) / 256 * a.n_labels >= 2 * 152 ? run(std::integral_constant<int, 2>{})
-                                                       : run(std::integral_constant<int, 1>{});
+        return (n + 255) / 256 * a.n_labels >= 2 * a.n_sm ? run(std::integral_constant<int, 2>{})
+                                                          : run(std::integral_constant<int, 1>{});
     });
     if (e != cudaSuccess || a.T_out || (!a.post && a.mode != CS_MODE_FACTORISED)) return e;
     const long long blocks = (n + 255) / 256;
-    normalise_plain_kernel<<<(unsigned)(blocks < 152 * 16 ? (blocks < 1 ? 1 : blocks) : 152 * 16), 256,
-                             0, st>>>(a);
+    normalise_plain_kernel<<<(unsigned)(blocks < most ? (blocks < 1 ? 1 : blocks) : most), 256, 0,
+                             st>>>(a);
     return cudaGetLastError();
 }
