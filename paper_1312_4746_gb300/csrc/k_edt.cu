@@ -6,8 +6,8 @@
 //   1. seed bitmaps: one bit per pixel and label;
 //   2. row pass (one warp per label and row): horizontal distance h to the
 //      nearest seed in the same row, from bit scans of the bitmap words;
-//   3. column pass (2 to 6 builder threads per label and column, one per
-//      row segment, and 8 to 32 readers): lower envelopes of the parabolas
+//   3. column pass (2 to 8 builder threads per label and column, one per
+//      row segment, and 8 or 32 readers): lower envelopes of the parabolas
 //      (y - q)^2 + h(q)^2 over each segment's rows q with finite h, each
 //      built in one sweep and read back by row ranges; intersection
 //      abscissae are compared as exact rationals with 64-bit cross products,
@@ -363,21 +363,22 @@ cudaError_t launch_edt(const EdtArgs& a, cudaStream_t st) {
         return cudaSuccess;
     };
     using std::integral_constant;
-    // Measured, the transform's three launches, us, columns per block / segments:
-    //                  columns   8/6   8/8  16/4  32/2  32/3
-    //   481 x 321 x 5     2405    44    46    50    67    58
-    //   640 x 480 x 5     3200    54    60    65    96    83
-    //   2000 x 200 x 3    6000    42    46    40    42    42
-    //   640 x 480 x 10    6400    86    93    67    95    87
-    //   3000 x 400 x 4   12000   116   129   115   141   128
-    //   481 x 321 x 30   14430    76    88    69    77    78
-    //   2000 x 200 x 8   16000    65    75    55    46    48
-    //   1024 x 1024 x 32 32768   518   639   386   345   321
-    //   23000 x 64 x 2   46000   239   249   218   208   211
-    e = ncol < 6000    ? run(integral_constant<int, 6>{}, integral_constant<int, 8>{})
-        : a.H <= 256   ? run(integral_constant<int, 2>{}, integral_constant<int, 32>{})
-        : ncol < 16000 ? run(integral_constant<int, 4>{}, integral_constant<int, 16>{})
-                       : run(integral_constant<int, 3>{}, integral_constant<int, 32>{});
+    // Measured, the transform's launches alone, us, columns per block / segments, on
+    // brush strokes of 60 and of 2000 samples per label (a label's rows are then few,
+    // and segments without seeds idle):
+    //                    columns   8/6       8/8       32/2      32/4
+    //   60 x 2000 x 5        300   82, 148   84, 134   177, 316  180, 300
+    //   481 x 321 x 5       2405   36, 42    37, 44    46, 72    48, 62
+    //   2000 x 200 x 5     10000   52, 63    58, 68    44, 60    47, 56
+    //   640 x 480 x 16     10240   63, 81    68, 84    74, 102   70, 102
+    //   1024 x 768 x 10    10240   102, 153  112, 156  102, 181  100, 151
+    //   1024 x 1024 x 16   16384   190, 285  212, 290  145, 211  142, 199
+    //   5000 x 100 x 5     25000   77, 85    81, 91    52, 61    56, 62
+    //   3000 x 400 x 16    48000   213, 292  241, 315  210, 325  204, 273
+    e = ncol >= 6000 && a.H <= 256   ? run(integral_constant<int, 2>{}, integral_constant<int, 32>{})
+        : ncol >= 16000              ? run(integral_constant<int, 4>{}, integral_constant<int, 32>{})
+        : ncol < 4000 && a.H > 1536  ? run(integral_constant<int, 8>{}, integral_constant<int, 8>{})
+                                     : run(integral_constant<int, 6>{}, integral_constant<int, 8>{});
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

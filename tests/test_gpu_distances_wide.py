@@ -1,8 +1,9 @@
-"""The distance transform's column pass by the number of columns (labels x width):
-8 columns per block below 6000, else 32 (at most 256 rows, or 16000 columns on) or 16;
-at the edges of that rule and of each form's shared memory (stacks of 440, 880 and 1758
-rows), with a last block that is not full and rows that the segments don't share
-evenly: exact integers, equal to the oracle's brute force.
+"""The distance transform's column pass by the number of columns (labels x width): 8
+columns per block and 6 segments (8 in tall narrow images), or 32 columns and 2 segments
+(from 6000 columns on, at most 256 rows) or 4 (from 16000 on); at the edges of that rule
+and of each form's shared memory (stacks of 440, 1758 and 1760 rows), with a last block
+that is not full and rows that the segments don't share evenly: exact integers, equal to
+the oracle's brute force.
 """
 import numpy as np
 import pytest
@@ -14,17 +15,17 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("H,W,m", [
     (66, 5999, [2]),           # 8 columns, 6 segments
-    (1758, 13, [3]),           # the same, the tallest in shared memory
-    (1759, 13, [3]),
     (59, 6000, [5]),           # 32 columns, 2 segments
     (256, 3001, [1, 3]),
-    (257, 3001, [1, 3]),       # 16 columns, 4 segments
-    (880, 2003, [1, 1, 2]),    # the tallest in shared memory
-    (881, 2003, [1, 1, 2]),
-    (261, 15999, [4]),         # the last before 32 columns, 3 segments
-    (261, 16001, [4]),
-    (438, 5347, [1, 1, 1]),    # the tallest in shared memory
-    (439, 5347, [1, 1, 1]),
+    (257, 3001, [1, 3]),       # 8 columns again
+    (261, 15999, [4]),
+    (261, 16001, [4]),         # 32 columns, 4 segments
+    (440, 5347, [1, 1, 1]),    # the tallest in shared memory
+    (441, 5347, [1, 1, 1]),
+    (1536, 13, [3, 2]),        # 8 columns, 6 segments
+    (1537, 13, [3, 2]),        # 8 segments
+    (1758, 2001, [1, 2]),      # 6 segments, the tallest in shared memory
+    (1759, 2001, [1, 2]),
 ])
 def test_column_forms(cuda_lib, H, W, m):
     import torch
