@@ -57,7 +57,7 @@ typedef int cs_status;
 
 /* Arithmetic forms. */
 #define CS_FP32 0 /* CUDA-core FP32 with exact integer distances; the TSM, an exact integer, from
-                     the tensor cores */
+                     the tensor cores, or from population counts for few samples per label */
 #define CS_BF16 1 /* tensor-core (tcgen05) TSM, colour and location dot products, FP32 accumulation */
 #define CS_FP8 2  /* as CS_BF16 with FP8 operands where they are exact */
 

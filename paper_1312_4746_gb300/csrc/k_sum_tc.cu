@@ -211,15 +211,17 @@ struct Cfg {
     static constexpr int EPQ = PAIR ? 2 : 4;                 // epilogue warps per TMEM lane quadrant
     static constexpr int EPI_WARPS = 4 * EPQ;
     static constexpr int CPW = BN / EPQ;                     // columns per epilogue warp per tile
-    // Producer warps. The sum's time follows its instructions, and a row of 32
-    // samples costs a producer about as much in waits and loop as in
-    // arithmetic: two warps per CTA form two rows each of a tile. Against four
-    // warps, with the registers this frees taken by the epilogue's loads in
-    // flight and the packed chunk sums: 481 x 321 412 -> 404 us, 1024 x 1024
-    // 36.5 -> 35.5 ms, 333 x 247 factorised 196 -> 189 us. One warp is faster
-    // still by up to 2% where location rows are truncations (402 us, 35.0 ms), but
-    // where they aren't (sides above LOC_NARROW) it holds the MMAs up: 3000 x 400,
-    // BF16, 3.59 ms against 3.21 with two and 3.39 with four.
+    // Producer warps. No unit of the kernel is full (issue 61 to 63%, ex2 54%, tensor
+    // 39%): its warps wait, for the packed chains' latencies, the tensor-memory loads
+    // and the ex2 queue. A row of 32 samples costs a producer about as much in waits
+    // and loop as in arithmetic, so two warps per CTA form two rows each of a tile.
+    // Against four warps, with the registers this frees taken by the epilogue's loads
+    // in flight and the packed chunk sums, the whole data term: 481 x 321 412 -> 408
+    // us, 1024 x 1024 36.5 -> 35.7 ms, 333 x 247 factorised 196 -> 189 us. One warp is
+    // faster still by up to 2% where location rows are truncations, but where they
+    // aren't (sides above LOC_NARROW) it holds the MMAs up: 3000 x 400, BF16, 3.59 ms
+    // against 3.21 with two and 3.39 with four; 4096 x 4096, 16 labels, FP8: 0.316 s
+    // with two, 0.325 with four.
     static constexpr int NPROD = 2;
     static constexpr int PRODUCER = EPI_WARPS;
     static constexpr int MMA_WARP = EPI_WARPS + NPROD;
